@@ -299,7 +299,9 @@ int sg_inner_cluster(const sg_problem* h);
  * 2 the cluster solver with the finest grid in global memory and the coarse
  * grids in shared memory (two blocks per SM, for batches too wide for 1).
  * After sg_autotune, the solver it timed fastest for that width (one of those
- * eligible); else the first eligible of 3, 1, 2, then 0.
+ * eligible); else the first eligible of 3, 1, 2, then 0. Path 0 includes the
+ * block-per-column solver of small grids (one launch per solve; off on a
+ * handle created while SGHSC_NO_BLOCK was 1).
  * h NULL or w <= 0: 0. */
 int sg_inner_path(const sg_problem* h, int w, int dtype);
 

@@ -2009,6 +2009,8 @@ int inner_solve(sg_problem* h, int dtype, const void* src, int ld_src, int src_t
   if (w <= 0) return SG_OK;
   if (o.m0 == SG_M0_VCYCLE && cluster_usable(h, dtype, w))
     return inner_solve_cluster(h, src, ld_src, src_t, dst, ld_dst, dst_t, w, o, s);
+  if (block_usable(h, dtype, w, o))
+    return inner_solve_block(h, dtype, src, ld_src, src_t, dst, ld_dst, dst_t, w, o, s);
   SG_TRY(ensure_inner_work(h, dtype, std::max(w, h->wmax)));
   if (dtype == SG_F64) return inner_solve_t<double>(h, src, ld_src, src_t, dst, ld_dst, dst_t, w, o, s);
   return inner_solve_t<float>(h, src, ld_src, src_t, dst, ld_dst, dst_t, w, o, s);

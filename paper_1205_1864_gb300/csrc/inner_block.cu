@@ -1,0 +1,724 @@
+// K3 + K4 on small grids: the batched inner PCG on A_0, one launch per solve,
+// every column solved by its own thread block (or cluster of blocks).
+//
+// Same method, stopping rule, status bits and iteration counts as the
+// stand-alone kernels of inner.cu. There an iteration is four to six launches
+// inside a graph WHILE node, about 45 us whatever the grid; on the paper's
+// own meshes (5 to 30 elements a side, FP64, some 50 iterations of the
+// diagonal M_0 per solve) that was all of the time. Here the loop is inside
+// the kernel and the column's vectors stay on chip:
+//
+//   k_block_diag    M_0 = diag(A_0), any grid of the Q1 stencil. A column is
+//                   split by rows over the C blocks of a cluster; each thread
+//                   keeps its nodes' stencil, r, p, x in registers, p with its
+//                   ghost rows in shared memory. Two cluster barriers per
+//                   iteration (p.q, then r.r with r.z): the neighbours' rows of
+//                   q travel with the first one, and each block carries r and
+//                   p of its ghost rows along itself.
+//   k_block_vcycle  M_0 = one V-cycle, finest grid of at most 1024 nodes: one
+//                   block per column, all grids in shared memory with zero
+//                   borders (no boundary tests in the stencils).
+//
+// What bounds them: the FP64 unit of each SM quarter takes a warp instruction
+// every 69 clocks (measured; one at a time, whatever the number of active
+// lanes or independent operands), so an iteration costs 69 clocks for every
+// FP64 instruction in the longest chain of one warp: the node's own sixteen,
+// then one for each step of a sum, and about eight for a division; a cluster
+// barrier adds 370 clocks. The blocks therefore use four warps where they can
+// (one per quarter), C is the largest split for which the batch still finds
+// an SM for every block, and every addition saved counts.
+//
+// Measured against the stand-alone kernels, sg_inner_solve with its copies
+// and synchronisation, 20 steps of the diagonal M_0 or 2 of the V-cycle:
+// 29 x 29 nodes, FP64, 20 columns 1412 -> 159 us, 1000 columns 4584 -> 1029;
+// 63 x 63, FP64, 300 columns 2833 -> 1503; 9 x 9, 20 columns 1487 -> 143;
+// V-cycle 15 x 15, FP64, 20 columns 251 -> 104, 31 x 31, FP32, 300 columns
+// 229 -> 120. No size it can hold was slower (1 to 1000 columns, both
+// types), so every batch that fits takes it. Whole FP64 solves: 16 x 16
+// elements, M = 3, p = 3, 6.64 -> 1.75 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
+// 274 -> 15.4 ms; lognormal 10 x 10, M = 3, p = 3, 1034 -> 77.6 ms.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "sghsc_internal.cuh"
+#include "vec.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace sghsc {
+
+namespace blk {
+constexpr int NT = 256;          // threads of k_block_diag at most
+constexpr int NW = NT / 32;
+constexpr int MAX_ITEMS = 4;     // nodes per thread of k_block_diag
+constexpr int MAX_C = 8;         // blocks per cluster
+constexpr int VNT = 256;         // threads of k_block_vcycle at most
+constexpr int MAX_GRIDS = 8;     // grids from 31 x 31 (or less) down to one node
+}  // namespace blk
+
+struct BlockArgs {
+  int n, nx, ny, w;
+  int R, C;            // k_block_diag: rows per block, blocks per column
+  double tol2;
+  int maxit, fixed;
+  int* status;
+  long long* iacc;
+  int* iters;          // per-column iteration counts, or null
+};
+
+// CG scalars of the block's column; every block of a cluster holds the same.
+template <typename T>
+struct BlockScalars {
+  double rho, stop;   // r.z of the last step; the r.r at which the column is done
+  T alpha, beta;
+  int it, done;
+};
+
+// The scalar updates of the stand-alone finaliser (col_update in inner.cu),
+// by one thread; report: this block writes status bits and counts.
+__device__ __forceinline__ bool is_nan_bits(long long b) {
+  return (b & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+}
+// x > 0 (false for NaN) and x <= y for non-negative y (false for a NaN x),
+// from the bit patterns: a comparison on the FP64 unit costs as much as a
+// multiply-add
+__device__ __forceinline__ bool positive(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool at_most(double x, double y) {
+  const long long b = __double_as_longlong(x), c = __double_as_longlong(y);
+  return b <= c && !is_nan_bits(b) && c <= 0x7ff0000000000000LL;
+}
+template <typename T>
+__device__ __forceinline__ void scal_init(BlockScalars<T>& S, double bb, const BlockArgs& a) {
+  S.stop = a.tol2 * bb;
+  S.done = !positive(bb);
+  S.it = 0;
+}
+template <typename T>
+__device__ __forceinline__ void scal_rho(BlockScalars<T>& S, double s) {
+  S.beta = (T)(S.it == 0 ? 0.0 : s / S.rho);
+  S.rho = s;
+}
+template <typename T>
+__device__ __forceinline__ void scal_alpha(BlockScalars<T>& S, double s, const BlockArgs& a, bool report) {
+  if (!positive(s)) {
+    if (report) atomicOr(a.status, ST_INNER_NOT_SPD);
+    S.alpha = T(0);
+    S.done = 1;
+  } else {
+    S.alpha = (T)(S.rho / s);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void scal_conv(BlockScalars<T>& S, double s, const BlockArgs& a, bool report) {
+  const int it = ++S.it;
+  bool fin;
+  if (a.fixed > 0) {
+    fin = it >= a.fixed;
+  } else {
+    fin = at_most(s, S.stop);
+    if (!fin && it >= a.maxit) {
+      fin = true;
+      if (report) atomicOr(a.status, ST_INNER_MAXIT);
+    }
+  }
+  if (is_nan_bits(__double_as_longlong(s))) {   // non-finite residual: stop the column and flag it
+    fin = true;
+    if (report) atomicOr(a.status, ST_INNER_NOT_SPD);
+  }
+  S.done = fin;
+  if (fin && report) {
+    atomicAdd((unsigned long long*)&a.iacc[0], (unsigned long long)it);
+    atomicMax(&a.iacc[1], (long long)it);
+  }
+}
+
+// Butterfly sum over the warp (every lane gets it).
+template <typename T>
+__device__ __forceinline__ T warp_sum(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The sums of v0 and v1 over the warp for the additions of one: lanes below
+// 16 end with the sum of v0, the others with that of v1.
+template <typename T>
+__device__ __forceinline__ T half_sums(T v0, T v1, int lane) {
+  const bool lo = lane < 16;
+  T v = lo ? v0 : v1;
+  v += __shfl_xor_sync(0xffffffffu, lo ? v1 : v0, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// ------------------------------------------------------- diagonal M_0 ---
+
+// Dynamic shared memory: p with ghost rows and columns [(R + 2)(nx + 2)],
+// then per ghost row side (above, below) q as received, r, dinv [2][nx] each.
+template <typename T>
+static size_t diag_smem(int R, int nx) {
+  return ((size_t)(R + 2) * (nx + 2) + 6 * (size_t)nx) * sizeof(T);
+}
+
+template <typename TS, typename T, typename TD, int ITEMS>
+__global__ void __launch_bounds__(blk::NT) k_block_diag(BlockArgs a, const T* __restrict__ st,
+                                                        const T* __restrict__ dinv, const TS* __restrict__ src,
+                                                        int lds, TD* __restrict__ dst, int ldd) {
+  using namespace blk;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ T red[3][MAX_C * NW];   // warp sums of every block of the cluster: r.r, r.z, p.q
+  __shared__ BlockScalars<T> S;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0;
+  const int col = blockIdx.x / C;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nx = a.nx, W = nx + 2;
+  const int r0 = rank * a.R, nr = max(0, min(a.ny - r0, a.R)), own = nr * nx;
+  T* ps = reinterpret_cast<T*>(smem_raw);
+  T* qg = ps + (size_t)(a.R + 2) * W;
+  T* rg = qg + 2 * nx;
+  T* dg = rg + 2 * nx;
+  const bool above = C > 1 && nr > 0 && r0 > 0, below = C > 1 && nr > 0 && r0 + nr < a.ny;
+  const int nt = blockDim.x, nw = nt / 32;
+  auto barrier = [&]() {
+    if (C > 1) cl.sync();
+    else __syncthreads();
+  };
+  auto put = [&](int k, int to, T v) {   // this warp's sum into slot k of block `to` of the cluster
+    T* s = &red[k][rank * nw + warp];
+    if (C > 1) *cl.map_shared_rank(s, to) = v;
+    else *s = v;
+  };
+  // warp sums into every block of the cluster: one sum, or two at the price
+  // of one (half a warp each; FP64 additions are what the sums cost)
+  auto push = [&](int k, T v) {
+    v = warp_sum(v);
+    if (lane < C) put(k, lane, v);
+  };
+  auto push2 = [&](T v0, T v1) {
+    const T s = half_sums(v0, v1, lane);
+    if ((lane & 15) < C) put(lane >> 4, lane & 15, s);
+  };
+  // totals, by one warp in a fixed order
+  const int ns = C * nw;   // warp sums per slot
+  auto total = [&](int k) {
+    T v = lane < ns ? red[k][lane] : T(0);
+    if (ns > 32) v += lane + 32 < ns ? red[k][lane + 32] : T(0);
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < ns) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return (double)v;
+  };
+  auto total2 = [&](double& s0, double& s1) {
+    const int l16 = lane & 15;
+    T v = l16 < ns ? red[lane >> 4][l16] : T(0);
+    for (int i = l16 + 16; i - l16 < ns; i += 16) v += i < ns ? red[lane >> 4][i] : T(0);
+    for (int o = 8; o > 0; o >>= 1)
+      if (o < ns) v += __shfl_xor_sync(0xffffffffu, v, o);
+    s0 = (double)__shfl_sync(0xffffffffu, v, 0);
+    s1 = (double)__shfl_sync(0xffffffffu, v, 16);
+  };
+  for (int i = tid; i < (a.R + 2) * W; i += nt) ps[i] = T(0);
+  T s9[ITEMS][9], r[ITEMS], x[ITEMS], z[ITEMS], d[ITEMS], q[ITEMS], p[ITEMS];
+  int pc[ITEMS];   // padded index
+  bool up[ITEMS], dn[ITEMS];   // node of the first / last own row, which a neighbour keeps as a ghost
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u) {
+    const int i = tid + u * nt;
+    const bool in = i < own;
+    const int ly = in ? i / nx : 0, lx = in ? i - ly * nx : 0, g = (r0 + ly) * nx + lx;
+    pc[u] = (ly + 1) * W + lx + 1;
+    up[u] = in && ly == 0 && above;
+    dn[u] = in && ly == nr - 1 && below;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) s9[u][e] = in ? st[(size_t)g * 9 + e] : T(0);
+    d[u] = in ? dinv[g] : T(0);
+    r[u] = in ? widen<T>(src[(size_t)g * lds + col]) : T(0);
+    x[u] = p[u] = q[u] = T(0);
+  }
+  for (int i = tid; i < 2 * nx; i += nt) {
+    const int side = i / nx, lx = i - side * nx, g = (side ? r0 + nr : r0 - 1) * nx + lx;
+    const bool in = side ? below : above;
+    rg[i] = in ? widen<T>(src[(size_t)g * lds + col]) : T(0);
+    dg[i] = in ? dinv[g] : T(0);
+  }
+  {
+    T rr = T(0), rz = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      z[u] = d[u] * r[u];
+      rr += r[u] * r[u];
+      rz += r[u] * z[u];
+    }
+    if (C > 1) cl.sync();   // every block of the cluster has started
+    push2(rr, rz);
+  }
+  barrier();
+  if (warp == 0) {
+    double bb, rz;
+    total2(bb, rz);
+    if (lane == 0) {
+      scal_init(S, bb, a);
+      if (!S.done) scal_rho(S, rz);
+    }
+  }
+  __syncthreads();
+  while (!S.done) {
+    const T beta = S.beta;
+    const bool first = S.it == 0;
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      if (tid + u * nt < own) {
+        p[u] = first ? z[u] : fma(beta, p[u], z[u]);
+        ps[pc[u]] = p[u];
+      }
+    }
+    if (C > 1)
+      for (int i = tid; i < 2 * nx; i += nt) {
+        const int side = i >= nx, lx = i - side * nx;
+        if (side ? below : above) {
+          T* pg = ps + (side ? nr + 1 : 0) * W + lx + 1;
+          const T zv = dg[i] * rg[i];
+          *pg = first ? zv : fma(beta, *pg, zv);
+        }
+      }
+    __syncthreads();
+    T pq = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      if (tid + u * nt < own) {
+        T acc = T(0);
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+          for (int dx = -1; dx <= 1; ++dx) acc = fma(s9[u][(dy + 1) * 3 + dx + 1], ps[pc[u] + dy * W + dx], acc);
+        q[u] = acc;
+        pq = fma(p[u], acc, pq);
+        if (up[u]) cl.map_shared_rank(qg, rank - 1)[nx + pc[u] - W - 1] = acc;
+        if (dn[u]) cl.map_shared_rank(qg, rank + 1)[pc[u] - nr * W - 1] = acc;
+      }
+    }
+    push(2, pq);
+    barrier();
+    if (warp == 0) {
+      const double s = total(2);
+      if (lane == 0) scal_alpha(S, s, a, rank == 0);
+    }
+    __syncthreads();
+    if (S.done) break;   // the same in every block of the cluster
+    const T al = S.alpha;
+    T rr = T(0), rz = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      if (tid + u * nt < own) {
+        x[u] = fma(al, p[u], x[u]);
+        r[u] = fma(-al, q[u], r[u]);
+        z[u] = d[u] * r[u];
+        rr = fma(r[u], r[u], rr);
+        rz = fma(r[u], z[u], rz);
+      }
+    }
+    if (C > 1)
+      for (int i = tid; i < 2 * nx; i += nt) rg[i] = fma(-al, qg[i], rg[i]);
+    push2(rr, rz);
+    barrier();
+    if (warp == 0) {
+      double s, rzs;
+      total2(s, rzs);
+      if (lane == 0) {
+        scal_conv(S, s, a, rank == 0);
+        if (!S.done) scal_rho(S, rzs);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u) {
+    const int i = tid + u * nt;
+    if (i < own) {
+      const int ly = i / nx, lx = i - ly * nx;
+      dst[(size_t)((r0 + ly) * nx + lx) * ldd + col] = (TD)x[u];
+    }
+  }
+  if (a.iters && rank == 0 && tid == 0) a.iters[col] = S.it;
+  if (C > 1) cl.sync();   // no block leaves while another may still store into it
+}
+
+// ---------------------------------------------------------- V-cycle M_0 ---
+
+// The hierarchy in shared memory: per grid (nx = ny = 2^k - 1, row stride
+// W = nx + 2) the vectors b, x, y with zero borders, the stencils [n][9] and
+// the inverse diagonal [n]; on the finest grid also p (with borders).
+struct BlockGrids {
+  int G;
+  int k[blk::MAX_GRIDS];                       // nx + 1 = 2^k
+  int vec[blk::MAX_GRIDS], coef[blk::MAX_GRIDS];   // element offsets of b (x, y follow) and of the stencils
+  int p, total;                                // offset of p, elements in all
+  const void* st[blk::MAX_GRIDS];
+  const void* dinv[blk::MAX_GRIDS];
+};
+
+// f(padded index, node) over the nodes of a grid of nx + 1 = 2^k, by the
+// threads t, t + nt, ... (columns of 2^k: the last of each row is skipped)
+template <typename F>
+__device__ __forceinline__ void each_node(int k, int t, int nt, F f) {
+  const int m = 1 << k, nx = m - 1;
+  for (int i = t; i < nx * m; i += nt) {
+    const int x = i & nx, y = i >> k;
+    if (x < nx) f((y + 1) * (m + 1) + x + 1, y * nx + x, x, y);
+  }
+}
+
+// acc + sign * (A v) at the node of padded index c
+template <int SIGN, typename T>
+__device__ __forceinline__ T dot9(T acc, const T* __restrict__ s9, const T* v, int c, int W) {
+#pragma unroll
+  for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+    for (int dx = -1; dx <= 1; ++dx) {
+      const T a = s9[(dy + 1) * 3 + dx + 1];
+      acc = fma(SIGN < 0 ? -a : a, v[c + dy * W + dx], acc);
+    }
+  return acc;
+}
+
+// Block barrier, or warp barrier while only warp 0 works (grids of at most 9
+// nodes).
+__device__ __forceinline__ void phase_sync(bool wm) {
+  if (wm) __syncwarp();
+  else __syncthreads();
+}
+
+// One V-cycle from the finest grid's b; returns the buffer that holds the
+// result. Every thread of the block calls it.
+template <typename T>
+__device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu) {
+  const int tid = threadIdx.x, G = L.G;
+  auto wmode = [&](int g) { return L.k[g] <= 2 && g > 0; };
+  auto vsize = [&](int g) { const int W = (1 << L.k[g]) + 1; return W * W; };
+  auto odd = [&](int s) { return (s & 1) != 0; };
+  // the iterate of grid g sits in x or y; pre-smoothing makes nu - 1 exchanges
+  for (int g = 0; g < G; ++g) {
+    const int W = (1 << L.k[g]) + 1, V = vsize(g), k = L.k[g], n = (W - 2) * (W - 2);
+    const bool wm = wmode(g);
+    const int nt = wm ? 32 : (int)blockDim.x;
+    const T* st = sm + L.coef[g];
+    const T* di = st + 9 * n;
+    const T* b = sm + L.vec[g];
+    T* c = sm + L.vec[g] + V;
+    T* o = c + V;
+    if (!wm || tid < 32) {
+      if (g == G - 1) {   // one node: exact
+        each_node(k, tid, nt, [&](int i, int node, int, int) { c[i] = di[node] * b[i]; });
+        phase_sync(wm);
+      } else {
+        each_node(k, tid, nt, [&](int i, int node, int, int) { c[i] = di[node] * b[i]; });
+        phase_sync(wm);
+        for (int s = 1; s < nu; ++s) {
+          each_node(k, tid, nt, [&](int i, int node, int, int) {
+            o[i] = fma(di[node], dot9<-1>(b[i], st + 9 * node, c, i, W), c[i]);
+          });
+          phase_sync(wm);
+          T* t = c; c = o; o = t;
+        }
+        each_node(k, tid, nt, [&](int i, int node, int, int) { o[i] = dot9<-1>(b[i], st + 9 * node, c, i, W); });
+        phase_sync(wm);
+        T* bc = sm + L.vec[g + 1];
+        each_node(L.k[g + 1], tid, nt, [&](int i, int, int X, int Y) {
+          const T* f = o + (2 * Y + 2) * W + 2 * X + 2;   // fine node (2X + 1, 2Y + 1)
+          T acc = T(0);
+#pragma unroll
+          for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+            for (int dx = -1; dx <= 1; ++dx)
+              acc += ((dx == 0 ? T(1) : T(0.5)) * (dy == 0 ? T(1) : T(0.5))) * f[dy * W + dx];
+          bc[i] = acc;
+        });
+        phase_sync(wm);
+      }
+    }
+  }
+  T* res = sm + L.vec[G - 1] + vsize(G - 1);
+  for (int g = G - 2; g >= 0; --g) {
+    const int W = (1 << L.k[g]) + 1, V = vsize(g), k = L.k[g], n = (W - 2) * (W - 2);
+    const int Wc = (1 << L.k[g + 1]) + 1;
+    const bool wm = wmode(g);
+    const int nt = wm ? 32 : (int)blockDim.x;
+    const T* st = sm + L.coef[g];
+    const T* di = st + 9 * n;
+    const T* b = sm + L.vec[g];
+    T* c = sm + L.vec[g] + V;
+    T* o = c + V;
+    if (odd(nu - 1)) { T* t = c; c = o; o = t; }
+    if (!wm && wmode(g + 1)) __syncthreads();   // results of warp 0
+    if (!wm || tid < 32) {
+      // bilinear interpolation: coarse node (X, Y) sits on fine (2X + 1, 2Y + 1);
+      // the zero border stands for the coarse nodes outside
+      const T* xc = res;
+      each_node(k, tid, nt, [&](int i, int, int x, int y) {
+        const int Xp = (x + 1) >> 1, Yp = (y + 1) >> 1;   // padded coarse index of the lower neighbour
+        const T* q = xc + Yp * Wc + Xp;
+        // weights 1 and 0 on odd coordinates, 1/2 and 1/2 on even ones: one
+        // chain for every parity (the lanes of a warp hold both)
+        const bool ox = x & 1, oy = y & 1;
+        const T w1 = ox ? T(0) : (oy ? T(0.5) : T(0.25)), w2 = oy ? T(0) : (ox ? T(0.5) : T(0.25));
+        const T w0 = ox ? (oy ? T(1) : T(0.5)) : (oy ? T(0.5) : T(0.25)), w3 = ox || oy ? T(0) : T(0.25);
+        // a zero weight reads the lower neighbour (the upper one may hold anything)
+        T v = fma(w0, q[0], c[i]);
+        v = fma(w1, q[ox ? 0 : 1], v);
+        v = fma(w2, q[oy ? 0 : Wc], v);
+        v = fma(w3, q[ox || oy ? 0 : Wc + 1], v);
+        c[i] = v;
+      });
+      phase_sync(wm);
+      for (int s = 0; s < nu; ++s) {
+        each_node(k, tid, nt, [&](int i, int node, int, int) {
+          o[i] = fma(di[node], dot9<-1>(b[i], st + 9 * node, c, i, W), c[i]);
+        });
+        phase_sync(wm);
+        T* t = c; c = o; o = t;
+      }
+    }
+    else if (odd(nu)) c = o;
+    res = c;
+  }
+  return res;
+}
+
+// Sum of v over the block, handed to f by one thread; ends with a barrier.
+template <typename T, typename F>
+__device__ __forceinline__ void block_sum(T* red, T v, F f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v = warp_sum(v);
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    const T s = warp_sum(lane < (int)(blockDim.x >> 5) ? red[lane] : T(0));
+    if (lane == 0) f((double)s);
+  }
+  __syncthreads();
+}
+
+template <typename TS, typename T, typename TD, int ITEMS>
+__global__ void __launch_bounds__(blk::VNT) k_block_vcycle(BlockArgs a, BlockGrids L, T om, int nu,
+                                                           const TS* __restrict__ src, int lds,
+                                                           TD* __restrict__ dst, int ldd) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ T red[blk::VNT / 32];
+  __shared__ BlockScalars<T> S;
+  T* sm = reinterpret_cast<T*>(smem_raw);
+  const int tid = threadIdx.x, NT = blockDim.x, col = blockIdx.x;
+  const int k = L.k[0], m = 1 << k, nx = m - 1, W = m + 1, V = W * W;
+  T* b = sm + L.vec[0];   // the residual is the V-cycle's right-hand side
+  T* ps = sm + L.p;
+  const T* st = sm + L.coef[0];
+  T x[ITEMS], q[ITEMS], p[ITEMS];
+  int pc[ITEMS], nd[ITEMS];
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u) {
+    const int i = tid + u * NT, xx = i & nx, y = i >> k;
+    const bool in = i < nx * m && xx < nx;
+    nd[u] = in ? y * nx + xx : -1;
+    pc[u] = in ? (y + 1) * W + xx + 1 : W + 1;
+    x[u] = p[u] = q[u] = T(0);
+  }
+  for (int g = 0; g < L.G; ++g) {
+    const int Wg = (1 << L.k[g]) + 1, ng = (Wg - 2) * (Wg - 2);
+    for (int i = tid; i < 3 * Wg * Wg; i += NT) sm[L.vec[g] + i] = T(0);
+    const T* gs = (const T*)L.st[g];
+    const T* gd = (const T*)L.dinv[g];
+    for (int i = tid; i < 9 * ng; i += NT) sm[L.coef[g] + i] = gs[i];
+    // the damped inverse diagonal (the plain one on the one-node grid, solved exactly)
+    for (int i = tid; i < ng; i += NT) sm[L.coef[g] + 9 * ng + i] = g == L.G - 1 ? gd[i] : om * gd[i];
+  }
+  for (int i = tid; i < V; i += NT) ps[i] = T(0);
+  __syncthreads();
+  {
+    T rr = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u)
+      if (nd[u] >= 0) {
+        const T v = widen<T>(src[(size_t)nd[u] * lds + col]);
+        b[pc[u]] = v;
+        rr += v * v;
+      }
+    block_sum(red, rr, [&](double s) { scal_init(S, s, a); });
+  }
+  while (!S.done) {
+    const T* z = block_vcycle<T>(L, sm, nu);   // ends with a block barrier
+    T rz = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u)
+      if (nd[u] >= 0) rz += b[pc[u]] * z[pc[u]];
+    block_sum(red, rz, [&](double s) { scal_rho(S, s); });
+    const T beta = S.beta;
+    const bool first = S.it == 0;
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u)
+      if (nd[u] >= 0) {
+        const T zv = z[pc[u]];
+        p[u] = first ? zv : zv + beta * p[u];
+        ps[pc[u]] = p[u];
+      }
+    __syncthreads();
+    T pq = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u)
+      if (nd[u] >= 0) {
+        q[u] = dot9<1>(T(0), st + 9 * nd[u], ps, pc[u], W);
+        pq = fma(p[u], q[u], pq);
+      }
+    block_sum(red, pq, [&](double s) { scal_alpha(S, s, a, true); });
+    if (S.done) break;
+    const T al = S.alpha;
+    T rr = T(0);
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u)
+      if (nd[u] >= 0) {
+        x[u] += al * p[u];
+        const T v = b[pc[u]] - al * q[u];
+        b[pc[u]] = v;
+        rr += v * v;
+      }
+    block_sum(red, rr, [&](double s) { scal_conv(S, s, a, true); });
+  }
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u)
+    if (nd[u] >= 0) dst[(size_t)nd[u] * ldd + col] = (TD)x[u];
+  if (a.iters && tid == 0) a.iters[col] = S.it;
+}
+
+// ------------------------------------------------------------ host side ---
+
+// Blocks per column of k_block_diag: as many (up to MAX_C) as leave an SM to
+// every block of the batch and at least two warps of nodes to each block, and
+// no fewer than hold the grid at MAX_ITEMS nodes a thread; 0 when that many
+// do not fit in a cluster.
+static int diag_split(const sg_problem* h, const GridLevel& G, int w) {
+  using namespace blk;
+  int C = 1;
+  while (C < MAX_C && (w * 2 * C <= h->num_sms) && G.n / (2 * C) >= 64 && G.ny >= 4 * C) C *= 2;
+  while (C <= MAX_C && ceil_div(G.ny, C) * G.nx > NT * MAX_ITEMS) C *= 2;
+  return C <= MAX_C && C <= G.ny ? C : 0;
+}
+
+static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L) {
+  L = BlockGrids{};
+  L.G = (int)h->grids.size();
+  if (!h->mg_full || L.G > blk::MAX_GRIDS || h->grids[0].n > 1024) return false;
+  int off = 0;
+  for (int g = 0; g < L.G; ++g) {
+    const GridLevel& G = h->grids[g];
+    int k = 0;
+    while ((1 << k) < G.nx + 1) ++k;
+    if (G.nx != G.ny || (1 << k) != G.nx + 1) return false;
+    L.k[g] = k;
+    L.vec[g] = off;
+    off += 3 * (G.nx + 2) * (G.nx + 2);
+    L.coef[g] = off;
+    off += 10 * G.n;
+    L.st[g] = es == 8 ? (const void*)G.st64 : (const void*)G.st32;
+    L.dinv[g] = es == 8 ? (const void*)G.dinv64 : (const void*)G.dinv32;
+  }
+  L.p = off;
+  off += (h->grids[0].nx + 2) * (h->grids[0].nx + 2);
+  L.total = off;
+  return (size_t)off * es <= (size_t)std::max(h->smem_optin, 48 * 1024) - 2048;
+}
+
+bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o) {
+  if (h->block_off || h->grids.empty() || w <= 0) return false;
+  const GridLevel& G = h->grids[0];
+  if (o.m0 == SG_M0_DIAG) {
+    const int C = diag_split(h, G, w);
+    const size_t es = dtype == SG_F64 ? 8 : 4;
+    return C > 0 && ((size_t)(ceil_div(G.ny, C) + 2) * (G.nx + 2) + 6 * (size_t)G.nx) * es <= 40 * 1024;
+  }
+  BlockGrids L;
+  return vcycle_layout(h, dtype == SG_F64 ? 8 : 4, L);
+}
+
+template <typename TS, typename T, typename TD>
+static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd, int w, const sg_prec_opts& o,
+                         cudaStream_t s) {
+  using namespace blk;
+  const GridLevel& G = h->grids[0];
+  const InnerWork& iw = sizeof(T) == 8 ? h->iw64 : h->iw32;
+  BlockArgs a;
+  a.n = G.n;
+  a.nx = G.nx;
+  a.ny = G.ny;
+  a.w = w;
+  a.C = a.R = 1;
+  a.tol2 = o.inner_tol * o.inner_tol;
+  a.maxit = o.inner_maxit;
+  a.fixed = o.inner_fixed_iters;
+  a.status = h->status;
+  a.iacc = h->iacc;
+  a.iters = iw.iters && iw.wcap >= w ? iw.iters : nullptr;
+  const T* st = sizeof(T) == 8 ? (const T*)G.st64 : (const T*)G.st32;
+  const T* dinv = sizeof(T) == 8 ? (const T*)G.dinv64 : (const T*)G.dinv32;
+  if (o.m0 == SG_M0_DIAG) {
+    a.C = diag_split(h, G, w);
+    a.R = ceil_div(G.ny, a.C);
+    // one warp per SM quarter (each has its own FP64 unit), more nodes a thread
+    // beyond that: a second warp would repeat the warp sums, not speed them up
+    const int nodes = a.R * G.nx;
+    const int threads = nodes > 128 * MAX_ITEMS ? NT : std::min(128, ceil_div(nodes, 32) * 32);
+    const int items = ceil_div(nodes, threads);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(w * a.C));
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = diag_smem<T>(a.R, G.nx);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = a.C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (items <= 1)
+      SG_TRY_CUDA(cudaLaunchKernelEx(&cfg, k_block_diag<TS, T, TD, 1>, a, st, dinv, src, lds, dst, ldd));
+    else if (items <= 2)
+      SG_TRY_CUDA(cudaLaunchKernelEx(&cfg, k_block_diag<TS, T, TD, 2>, a, st, dinv, src, lds, dst, ldd));
+    else
+      SG_TRY_CUDA(cudaLaunchKernelEx(&cfg, k_block_diag<TS, T, TD, 4>, a, st, dinv, src, lds, dst, ldd));
+    note_launch();
+    return SG_OK;
+  }
+  BlockGrids L;
+  if (!vcycle_layout(h, sizeof(T), L)) {
+    set_error("block inner solve: the hierarchy does not fit");
+    return SG_ERR_UNSUPPORTED;
+  }
+  const size_t smem = (size_t)L.total * sizeof(T);
+  auto go = [&](auto kern, int threads) -> int {
+    SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    { kern<<<w, threads, smem, s>>>(a, L, (T)o.omega, o.nu, src, lds, dst, ldd); note_launch(); }
+    SG_CHECK_LAUNCH();
+    return SG_OK;
+  };
+  if (G.nx <= 15) return go(k_block_vcycle<TS, T, TD, 2>, 128);
+  return go(k_block_vcycle<TS, T, TD, 4>, 256);
+}
+
+int inner_solve_block(sg_problem* h, int dtype, const void* src, int lds, int src_t, void* dst, int ldd, int dst_t,
+                      int w, const sg_prec_opts& o, cudaStream_t s) {
+  const bool s64 = src_t == SG_F64, d64 = dst_t == SG_F64;
+  if (dtype == SG_F64) {
+    if (s64 && d64) return solve_block_t<double, double, double>(h, (const double*)src, lds, (double*)dst, ldd, w, o, s);
+    set_error("block inner solve: FP64 solves take FP64 blocks");
+    return SG_ERR_UNSUPPORTED;
+  }
+  if (s64 && d64) return solve_block_t<double, float, double>(h, (const double*)src, lds, (double*)dst, ldd, w, o, s);
+  if (s64) return solve_block_t<double, float, float>(h, (const double*)src, lds, (float*)dst, ldd, w, o, s);
+  if (d64) return solve_block_t<float, float, double>(h, (const float*)src, lds, (double*)dst, ldd, w, o, s);
+  return solve_block_t<float, float, float>(h, (const float*)src, lds, (float*)dst, ldd, w, o, s);
+}
+
+}  // namespace sghsc

@@ -500,6 +500,8 @@ static int setup_impl(const sg_mesh* mesh, int M, int p, int family, int n, int 
   {
     const char* ev = getenv("SGHSC_NO_PIPE");
     h->pipe_off = ev && ev[0] == '1';
+    const char* eb = getenv("SGHSC_NO_BLOCK");
+    h->block_off = eb && eb[0] == '1';
   }
   {
     const char* ev = getenv("SGHSC_GATHER_FORM");   // start from the gather form of the full product

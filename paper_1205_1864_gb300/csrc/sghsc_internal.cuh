@@ -176,6 +176,7 @@ struct sg_problem {
   void* cl_plan = nullptr;                  // cluster inner solvers: plans and scratch (null: not usable)
   std::map<int, int> inner_pick;            // FP32 batch width -> inner solver chosen by the autotuner
   bool pipe_off = false;                    // SGHSC_NO_PIPE=1: no row-pipelined sweeps on large grids
+  bool block_off = false;                   // SGHSC_NO_BLOCK=1: no block-per-column inner solver on small grids
   // workspace
   sghsc::InnerWork iw32, iw64;
   float* R32 = nullptr;                     // n x P working residual (mixed HSC)
@@ -290,6 +291,13 @@ std::vector<int> inner_path_candidates(const sg_problem* h, int w);
 // inner_solve for FP32 on a usable handle: one cluster launch per solve.
 int inner_solve_cluster(sg_problem* h, const void* src, int ld_src, int src_t, void* dst, int ld_dst, int dst_t,
                         int w, const sg_prec_opts& o, cudaStream_t s);
+
+// ---- inner solver on small grids, one launch per solve (inner_block.cu) ----
+// Batches the cluster solver does not take: any grid that a cluster of
+// blocks holds with the diagonal M_0, at most 1024 nodes with the V-cycle.
+bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o);
+int inner_solve_block(sg_problem* h, int dtype, const void* src, int ld_src, int src_t, void* dst, int ld_dst,
+                      int dst_t, int w, const sg_prec_opts& o, cudaStream_t s);
 
 // ---- HSC / mean preconditioner (hsc.cu) ----
 int prepare_precond(sg_problem* h, int kind, const sg_prec_opts& o);
