@@ -26,7 +26,7 @@
 namespace sghsc {
 
 constexpr int DF_CH = 9;       // nonzeros per staged chunk (the Q1 stencil row)
-constexpr int DF_MAXQ = 12;    // pairs per thread kept in registers
+constexpr int DF_MAXQ = 12;    // pairs per thread and row at most
 
 // FP32 value of an input element that is FP32-exact: a float as it is, a
 // double (the FP64 widening of an FP32 number) re-packed with integer
@@ -54,24 +54,62 @@ __device__ __forceinline__ df64 df_mul_f(const df64& a, float x) {
   return df64(p, e);
 }
 
-// Row strides of the staged chunk: a term's nine values padded to ten
-// double-float slots (80 bytes: five 16-byte loads), an input column's nine
-// values padded to twelve floats (48 bytes: three 16-byte loads; a warp's
-// eight-lane phases of consecutive columns then hit distinct bank groups).
-constexpr int DF_VS = 10;
-constexpr int DF_XS = 12;
+// Packed FP32 operations (f32x2): two per instruction. The FP32 lanes are no
+// faster (38 T operations/s packed or not), but the arithmetic takes half the
+// issue slots, which the addresses, loads and integer work share. Measured with
+// the packed sums and couplings (and the order of the couplings chosen against
+// bank conflicts in setup.cu) against the scalar form: full product 255^2,
+// M = 10, p = 4 2.54 -> 2.43 ms, 200^2, M = 8, p = 4 0.711 -> 0.691; level
+// products 255^2, M = 10, 715 -> 220 columns 1.04 -> 0.99, M = 4, 20 <-> 35
+// columns 0.247 -> 0.200, 10 <- 55 columns 0.290 -> 0.236; the even and odd
+// partial sums halve the error against 64 bits (9.8e-15 -> 4.9e-15). Also
+// tried: two sums per lane sharing the term's values, the next row prefetched
+// into registers, half of a block's warps coupling while the others sum (2.6 to
+// 2.8 ms each at M = 10, p = 4): the sums alone, in registers, run at 0.75 of
+// the lanes' rate, and staging, couplings and conversions each need issue slots
+// that a second role on the same SM does not find free.
+struct df64x2 {   // two double-float values
+  float2 hi, lo;
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }   // folds into the operand
 
-// Stage chunk cs..cs+nzc-1 (nzc <= DF_CH): values [k][e], inputs [j][e],
-// slots e >= nzc zero. The input rows go column position by column position
-// (no integer division), the loads of all slots of a position in flight
-// before their 16-byte stores.
+// the products of a.hi and x exactly, plus lo (a.lo x)
+__device__ __forceinline__ df64x2 df_mul_f2(float2 hi, float2 lo, float2 x) {
+  df64x2 r;
+  r.hi = __fmul2_rn(hi, x);
+  r.lo = __ffma2_rn(lo, x, __ffma2_rn(hi, x, neg2(r.hi)));
+  return r;
+}
+// s += v: two-sum of the hi parts, the lo parts in FP32
+__device__ __forceinline__ void df_add2(df64x2& s, const df64x2& v) {
+  const float2 t = __fadd2_rn(s.hi, v.hi);
+  const float2 bb = __fadd2_rn(t, neg2(s.hi));
+  const float2 e = __fadd2_rn(__fadd2_rn(s.hi, neg2(__fadd2_rn(t, neg2(bb)))), __fadd2_rn(v.hi, neg2(bb)));
+  s.hi = t;
+  s.lo = __fadd2_rn(__fadd2_rn(s.lo, v.lo), e);
+}
+
+// Layout of the staged chunk (DF_VS, DF_XS: sghsc_internal.cuh, the setup packs
+// the pairs' offsets). A term's nine double-float values: eight hi parts,
+// eight lo parts (neighbouring nonzeros side by side for the packed
+// operations), then the ninth pair. An input column's nine values, padded to
+// 12 floats: the eight lanes of a 16-byte load phase of consecutive columns
+// then hit distinct banks.
+
+// Stage chunk cs..cs+nzc-1 (nzc <= DF_CH), slots e >= nzc zero. The input rows
+// go column position by column position (no integer division), the loads of
+// all slots of a position in flight before their 16-byte stores.
 template <typename TX>
 __device__ __forceinline__ void df_stage(int cs, int nzc, int M1, const int* __restrict__ colidx,
                                          const df64* __restrict__ vals, const TX* __restrict__ X, int ldx, int wx,
-                                         df64* Vt, float* Xt) {
+                                         float* Vt, float* Xt) {
   for (int k = threadIdx.x; k < M1; k += blockDim.x) {
 #pragma unroll
-    for (int e = 0; e < DF_VS; ++e) Vt[k * DF_VS + e] = e < nzc ? vals[(size_t)(cs + e) * M1 + k] : df64(0.f, 0.f);
+    for (int e = 0; e < DF_CH; ++e) {
+      const df64 v = e < nzc ? vals[(size_t)(cs + e) * M1 + k] : df64(0.f, 0.f);
+      Vt[k * DF_VS + (e < 8 ? e : 16)] = v.hi;
+      Vt[k * DF_VS + (e < 8 ? 8 + e : 17)] = v.lo;
+    }
   }
   int col[DF_CH];
 #pragma unroll
@@ -88,26 +126,33 @@ __device__ __forceinline__ void df_stage(int cs, int nzc, int M1, const int* __r
 }
 
 // sum_e a[e] x[e] over the DF_CH slots of one staged term row and one staged
-// input column, both read as 16-byte vectors
-__device__ __forceinline__ df64 df_dot9(const df64* __restrict__ a, const float* __restrict__ x) {
-  const float4* av = reinterpret_cast<const float4*>(a);   // two double-float values each
+// input column: the even and odd slots in packed sums, then the two halves
+// added and the ninth slot.
+__device__ __forceinline__ df64 df_dot9(const float* __restrict__ a, const float* __restrict__ x) {
+  const float4* av = reinterpret_cast<const float4*>(a);
   const float4* xv = reinterpret_cast<const float4*>(x);
-  const float4 x0 = xv[0], x1 = xv[1], x2 = xv[2];
-  float4 v = av[0];
-  df64 s = df_mul_f(df64(v.x, v.y), x0.x);
-  s += df_mul_f(df64(v.z, v.w), x0.y);
-  v = av[1];
-  s += df_mul_f(df64(v.x, v.y), x0.z);
-  s += df_mul_f(df64(v.z, v.w), x0.w);
-  v = av[2];
-  s += df_mul_f(df64(v.x, v.y), x1.x);
-  s += df_mul_f(df64(v.z, v.w), x1.y);
-  v = av[3];
-  s += df_mul_f(df64(v.x, v.y), x1.z);
-  s += df_mul_f(df64(v.z, v.w), x1.w);
-  v = av[4];
-  s += df_mul_f(df64(v.x, v.y), x2.x);
-  return s;
+  auto lo2 = [](const float4& v) { return make_float2(v.x, v.y); };
+  auto hi2 = [](const float4& v) { return make_float2(v.z, v.w); };
+  const float4 x0 = xv[0], x1 = xv[1], h0 = av[0], h1 = av[1], l0 = av[2], l1 = av[3];
+  const float2 t8 = *reinterpret_cast<const float2*>(a + 16);
+  const float x8 = x[8];
+  df64x2 s = df_mul_f2(lo2(h0), lo2(l0), lo2(x0));
+  df_add2(s, df_mul_f2(hi2(h0), hi2(l0), hi2(x0)));
+  df_add2(s, df_mul_f2(lo2(h1), lo2(l1), lo2(x1)));
+  df_add2(s, df_mul_f2(hi2(h1), hi2(l1), hi2(x1)));
+  df64 r(s.hi.x, s.lo.x);
+  r += df64(s.hi.y, s.lo.y);
+  r += df_mul_f(df64(t8.x, t8.y), x8);
+  return r;
+}
+
+// an FP32 number as FP64 (f2d_bits), the common case first: a normal number's
+// exponent rebiased and its fraction moved, five operations
+__device__ __forceinline__ double f2d_fast(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if (e - 1u < 254u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+  return f2d_bits(f);
 }
 
 enum { DF_SUB = 0, DF_PLAIN = 1, DF_OUTER = 2 };
@@ -128,7 +173,7 @@ enum { DF_SUB = 0, DF_PLAIN = 1, DF_OUTER = 2 };
 template <bool DIAG, int MODE, typename TX, typename TY, int LB>
 __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
     int n, const int* __restrict__ rowptr, const int* __restrict__ colidx, const df64* __restrict__ vals, int M1,
-    const TX* __restrict__ X, int ldx, int wx, int npair, const int* __restrict__ pk, const int* __restrict__ pj,
+    const TX* __restrict__ X, int ldx, int wx, int npair, const unsigned* __restrict__ pkj,
     const unsigned* __restrict__ ctr, const int2* __restrict__ sdesc, const df64* __restrict__ ctab, int ncls, int wy,
     const double* __restrict__ Yin, int ldyin, TY* __restrict__ Y, int ldy, double* pA, double* pB,
     double* __restrict__ q, OuterArgs a) {
@@ -138,19 +183,17 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
   // warp runs the same loops (the padding pairs read staged slot 0 and write
   // sums nothing reads)
   const int nq = (npair + LB - 1) / LB, nd = DIAG ? (wy + LB - 1) / LB : 0;
-  df64* Ss = reinterpret_cast<df64*>(smem_raw);
-  df64* Ds = Ss + (size_t)nq * LB;
-  df64* Ctab = Ds + (size_t)nd * LB;
-  df64* Vt = Ctab + ((ncls + 1) & ~1);
-  float* Xt = reinterpret_cast<float*>(Vt + (size_t)M1 * DF_VS);
-  for (int t = threadIdx.x; t < ncls; t += blockDim.x) Ctab[t] = ctab[t];
-  // this thread's pairs (consecutive threads: consecutive pairs), as the
-  // staged offsets of their term row and input column
-  unsigned qkj[DF_MAXQ];   // k DF_VS << 16 | j DF_XS
-#pragma unroll
-  for (int i = 0; i < DF_MAXQ; ++i) {
-    const int qi = threadIdx.x + i * blockDim.x;
-    qkj[i] = qi < npair ? ((unsigned)(pk[qi] * DF_VS) << 16) | (unsigned)(pj[qi] * DF_XS) : 0u;
+  // hi and lo parts apart: the packed coupling sums read them as they are
+  float* Sh = reinterpret_cast<float*>(smem_raw);
+  float* Sl = Sh + (size_t)nq * LB;
+  float* Dh = Sl + (size_t)nq * LB;
+  float* Dl = Dh + (size_t)nd * LB;
+  float* Vt = Dl + (size_t)nd * LB;
+  float* Xt = Vt + (size_t)M1 * DF_VS;
+  __shared__ float Ch[256], Cl[256];
+  for (int t = threadIdx.x; t < ncls; t += blockDim.x) {
+    Ch[t] = ctab[t].hi;
+    Cl[t] = ctab[t].lo;
   }
   int it = 0;
   double beta = 0.0, dot = 0.0;
@@ -173,47 +216,84 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
       if (DIAG) {
         for (int i = 0; i < nd; ++i) {
           const int l = threadIdx.x + i * LB;
-          const df64 d = df_dot9(Vt, Xt + min(l, wx - 1) * DF_XS);
-          if (first) Ds[l] = d; else Ds[l] += d;
+          df64 d = df_dot9(Vt, Xt + min(l, wx - 1) * DF_XS);
+          if (!first) d += df64(Dh[l], Dl[l]);
+          Dh[l] = d.hi;
+          Dl[l] = d.lo;
         }
       }
-#pragma unroll
-      for (int i = 0; i < DF_MAXQ; ++i) {
-        if (i < nq) {   // the same for the whole block
-          const int qi = threadIdx.x + i * LB;
-          const df64 s = df_dot9(Vt + (qkj[i] >> 16), Xt + (qkj[i] & 0xffffu));
-          if (first) Ss[qi] = s; else Ss[qi] += s;
-        }
+      // consecutive threads: consecutive pairs, each as its staged offsets
+      const unsigned* pp = pkj + threadIdx.x;
+      unsigned next = threadIdx.x < npair ? __ldg(pp) : 0u;
+#pragma unroll 2
+      for (int qi = threadIdx.x; qi < nq * LB; qi += LB) {
+        const unsigned o = next;
+        pp += LB;
+        next = qi + LB < npair ? __ldg(pp) : 0u;
+        df64 s = df_dot9(Vt + (o >> 16), Xt + (o & 0xffffu));
+        if (!first) s += df64(Sh[qi], Sl[qi]);
+        Sh[qi] = s.hi;
+        Sl[qi] = s.lo;
       }
     }
     __syncthreads();
     for (int slot = threadIdx.x; slot < wy; slot += LB) {
       const int2 d = __ldg(sdesc + slot);
       const int l = (int)((unsigned)d.y >> 16), ncl = d.y & 0xffff;   // ncl: the warp's count
-      df64 acc = (DIAG && re > rb) ? Ds[l] : df64(0.f, 0.f);
-      if (re > rb) {
-        const unsigned* cw = ctr + d.x;
-#pragma unroll 4
-        for (int c = 0; c < ncl; ++c) {
-          const unsigned w = __ldg(cw + 32 * c);
-          acc += Ctab[w & 0xffu] * Ss[w >> 8];
+      double zv = 0.0, po = 0.0, qo = 0.0, yin = 0.0;   // loaded before the sums that they meet
+      if constexpr (OUTER) {
+        const size_t g = (size_t)r * wx + l;
+        zv = widen_exact(X[g]);
+        if (it != 0) {
+          po = pold[g];
+          qo = q[g];
         }
+      }
+      if constexpr (MODE == DF_SUB) yin = Yin[(size_t)r * ldyin + l];
+      df64 acc(0.f, 0.f);
+      if (re > rb) {
+        if (DIAG) acc = df64(Dh[l], Dl[l]);
+        // two couplings at a time, side by side in packed sums; past the last
+        // one the zero coefficient class (word 0)
+        auto at = [](const float* p, unsigned byte) {
+          return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(p) + byte);
+        };
+        auto couple = [&](unsigned w0, unsigned w1, df64x2& s) {
+          const unsigned k0 = w0 & 0x3ffu, k1 = w1 & 0x3ffu, q0 = w0 >> 10, q1 = w1 >> 10;
+          const float2 ch = make_float2(at(Ch, k0), at(Ch, k1)), cl = make_float2(at(Cl, k0), at(Cl, k1));
+          const float2 sh = make_float2(at(Sh, q0), at(Sh, q1)), sl = make_float2(at(Sl, q0), at(Sl, q1));
+          df64x2 v;
+          v.hi = __fmul2_rn(ch, sh);
+          v.lo = __ffma2_rn(cl, sh, __ffma2_rn(ch, sl, __ffma2_rn(ch, sh, neg2(v.hi))));
+          df_add2(s, v);
+        };
+        const unsigned* cw = ctr + d.x;
+        df64x2 s;
+        s.hi = s.lo = make_float2(0.f, 0.f);
+        int c = 0;
+        for (; c + 4 <= ncl; c += 4, cw += 128) {
+          const unsigned w0 = __ldg(cw), w1 = __ldg(cw + 32), w2 = __ldg(cw + 64), w3 = __ldg(cw + 96);
+          couple(w0, w1, s);
+          couple(w2, w3, s);
+        }
+        for (; c < ncl; c += 2, cw += 64) couple(__ldg(cw), c + 1 < ncl ? __ldg(cw + 32) : 0u, s);
+        acc += df64(s.hi.x, s.lo.x);
+        acc += df64(s.hi.y, s.lo.y);
       }
       acc = df_norm(acc);
       if constexpr (OUTER) {
         const size_t g = (size_t)r * wx + l;
-        const double av = f2d_bits(acc.hi) + f2d_bits(acc.lo);
-        const double zv = widen_exact(X[g]);
-        const double pv = it == 0 ? zv : zv + beta * pold[g];
-        const double qv = it == 0 ? av : av + beta * q[g];
+        const double av = f2d_fast(acc.hi) + f2d_fast(acc.lo);
+        const double pv = it == 0 ? zv : zv + beta * po;
+        const double qv = it == 0 ? av : av + beta * qo;
         pnew[g] = pv;
         q[g] = qv;
         dot += pv * qv;
       } else if constexpr (MODE == DF_PLAIN) {
-        Y[(size_t)r * ldy + l] = f2d_bits(acc.hi) + f2d_bits(acc.lo);
+        Y[(size_t)r * ldy + l] = f2d_fast(acc.hi) + f2d_fast(acc.lo);
       } else {
         // Yin - sum in double-float, rounded once to FP32
-        df64 v = df_from_double(Yin[(size_t)r * ldyin + l]);
+        df64 v = df_from_double(yin);
         v += df64(-acc.hi, -acc.lo);
         Y[(size_t)r * ldy + l] = v.hi + v.lo;
       }
@@ -221,7 +301,10 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
   }
   if constexpr (OUTER) {
     double pq, unused;
-    if (outer_reduce_last(dot, 0.0, a, pq, unused) && threadIdx.x == 0) {
+    // (the sums' shared memory is free after the last row)
+    __syncthreads();
+    double* red = reinterpret_cast<double*>(smem_raw);
+    if (outer_reduce_last(dot, 0.0, a, pq, unused, red, red + LB) && threadIdx.x == 0) {
       a.sc[SC_PQ] = pq;
       if (!(pq > 0.0)) {
         atomicOr(a.status, ST_OUTER_BREAKDOWN);
@@ -238,19 +321,21 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
 // 512 (more, smaller blocks hide the row barriers better).
 static int df_threads(const EdgeList& E) { return E.npair <= DF_MAXQ * 256 ? 256 : 512; }
 
+// (at least the outer step's final sums of two doubles per thread)
 static size_t df_smem(const EdgeList& E, int M1, int wx, bool diag) {
   const size_t t = (size_t)df_threads(E);
   auto pad = [t](size_t v) { return (v + t - 1) / t * t; };
-  return (pad(E.npair) + (diag ? pad(E.nout) : 0) + ((E.ncls + 1) & ~1) + (size_t)M1 * DF_VS) * sizeof(df64) +
-         (size_t)wx * DF_XS * sizeof(float);
+  return std::max((2 * (pad(E.npair) + (diag ? pad(E.nout) : 0)) + (size_t)M1 * DF_VS + (size_t)wx * DF_XS) *
+                      sizeof(float),
+                  t * 2 * sizeof(double));
 }
 
 // Usable when every thread's pairs fit its registers, the couplings have a
 // compact table with slot descriptors and the staging fits a block's shared
 // memory.
 bool df_pairs_usable(const sg_problem* h, const EdgeList& E, int wx) {
-  return h->staged_pairs && E.npair <= DF_MAXQ * 512 && E.ncls > 0 && E.sdesc && h->nterm * DF_VS < 65536 &&
-         wx * DF_XS < 65536 && df_smem(E, h->nterm, wx, true) <= (size_t)std::max(h->smem_optin, 48 * 1024);
+  return h->staged_pairs && E.npair <= DF_MAXQ * 512 && (E.pkj || E.npair == 0) && E.ncls > 0 && E.sdesc && h->nterm * DF_VS < 65536 &&
+         wx * DF_XS < 65536 && df_smem(E, h->nterm, wx, true) + 4 * 1024 <= (size_t)std::max(h->smem_optin, 48 * 1024);
 }
 
 template <bool DIAG, int MODE, typename TX, typename TY>
@@ -268,7 +353,7 @@ static int launch_df(sg_problem* h, const EdgeList& E, const TX* X, int ldx, int
     int grid = std::min(h->n, h->num_sms * std::max(per_sm, 1));
     if (MODE == DF_OUTER) grid = std::min(grid, h->opart_blocks);
     { kern<<<grid, threads, smem, s>>>(h->n, h->rowptr, h->colidx, (const df64*)h->vals_df, h->nterm, X, ldx, wx,
-                                       E.npair, E.pk, E.pj, E.ctr, E.sdesc, (const df64*)E.ctab, E.ncls, wy, Yin,
+                                       E.npair, E.pkj, E.ctr, E.sdesc, (const df64*)E.ctab, E.ncls, wy, Yin,
                                        ldyin, Y, ldy, h->fpA, h->fpB, h->fq, a); ::sghsc::note_launch(); }
     SG_CHECK_LAUNCH();
     return SG_OK;

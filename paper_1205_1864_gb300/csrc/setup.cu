@@ -65,6 +65,67 @@ struct HostEdges {
   std::vector<double> c;
 };
 
+// The order in which the 32 output slots of a warp take their couplings, so
+// that the words a warp reads together lie in different shared-memory banks
+// (in list order a step's reads met up to eight deep in one bank). addr[s]:
+// word address of each coupling of slot s; row c of the result holds, per slot,
+// the index of the coupling taken at step c, or -1 (padding). As many rows as
+// the longest list. Greedy: at each step the slots with most left choose
+// first, the address that shares its bank with the fewest others; a slot with
+// steps to spare waits rather than collide.
+using WarpSchedule = std::vector<std::vector<int>>;
+static WarpSchedule schedule_warp(const std::vector<std::vector<int>>& addr) {
+  WarpSchedule w;
+  const int n = (int)addr.size();
+  size_t rows = 0;
+  std::vector<std::vector<int>> left(n);
+  std::vector<int> demand(32, 0);
+  for (int s = 0; s < n; ++s) {
+    rows = std::max(rows, addr[s].size());
+    for (int i = 0; i < (int)addr[s].size(); ++i) {
+      left[s].push_back(i);
+      ++demand[addr[s][i] & 31];
+    }
+  }
+  std::vector<int> order(n);
+  if (rows > 64) {   // the dense couplings of a gPC coefficient: list order (the search is quadratic)
+    for (size_t r = 0; r < rows; ++r) {
+      std::vector<int> take(n, -1);
+      for (int s = 0; s < n; ++s)
+        if (r < addr[s].size()) take[s] = (int)r;
+      w.push_back(take);
+    }
+    return w;
+  }
+  for (size_t r = 0; r < rows; ++r) {
+    std::vector<int> take(n, -1);
+    std::vector<std::vector<int>> bank(32);   // distinct addresses read so far
+    for (int s = 0; s < n; ++s) order[s] = s;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return left[a].size() > left[b].size(); });
+    for (int s : order) {
+      int best = -1, cost = 0;
+      for (int q = 0; q < (int)left[s].size(); ++q) {
+        const int a = addr[s][left[s][q]];
+        const auto& B = bank[a & 31];
+        const int c = std::count(B.begin(), B.end(), a) ? 0 : (int)B.size();
+        if (best < 0 || c < cost || (c == cost && demand[a & 31] > demand[addr[s][left[s][best]] & 31])) {
+          best = q;
+          cost = c;
+        }
+      }
+      if (best < 0 || (cost > 0 && left[s].size() < rows - r)) continue;
+      const int a = addr[s][left[s][best]];
+      auto& B = bank[a & 31];
+      if (!std::count(B.begin(), B.end(), a)) B.push_back(a);
+      --demand[a & 31];
+      take[s] = left[s][best];
+      left[s].erase(left[s].begin() + best);
+    }
+    w.push_back(take);
+  }
+  return w;
+}
+
 static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 = 0, int nin = 0) {
   E.out0 = out0;
   E.in0 = in0;
@@ -103,6 +164,15 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 
   for (int t = 0; t < E.nedges; ++t) pair[t] = pairs.at(std::make_pair(he.k[t], he.j[t]));
   E.npair = (int)pk.size();
   {
+    std::vector<unsigned> w(pk.size());
+    bool fits = true;
+    for (size_t q = 0; q < pk.size(); ++q) {
+      fits = fits && pk[q] * DF_VS < 65536 && pj[q] * DF_XS < 65536;
+      w[q] = ((unsigned)(pk[q] * DF_VS) << 16) | (unsigned)(pj[q] * DF_XS);
+    }
+    if (fits && pk.size() < (1u << 20)) SG_TRY(upload(&E.pkj, w.data(), w.size()));
+  }
+  {
     // coefficient classes; class 0 is the coefficient 0, which pads the
     // shorter slots of a warp to the warp's longest (a zero word adds 0)
     std::map<double, int> cls;
@@ -132,13 +202,25 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 
       const int wts = rows32_stride(nin);   // the row stride of the FP32 row kernel's term sums
       for (int t = 0; t < E.nedges; ++t) kj_ok = kj_ok && (long long)he.k[t] * wts + he.j[t] < (1 << 24);
       if (kj_ok) pkj.assign(packed.size(), 0u);
-      for (int sl = 0; sl < E.nout; ++sl) {
-        const int l = perm[sl];
-        for (int t = he.ptr[l]; t < he.ptr[l + 1]; ++t) {
-          const unsigned c = (unsigned)cls.at(he.c[t]);
-          packed[tb[sl] + 32 * (t - he.ptr[l])] = ((unsigned)pair[t] << 8) | c;
-          if (kj_ok) pkj[tb[sl] + 32 * (t - he.ptr[l])] = (c << 24) | (unsigned)(he.k[t] * wts + he.j[t]);
+      for (int w0 = 0; w0 < E.nout; w0 += 32) {
+        const int ws = std::min(32, E.nout - w0);
+        std::vector<std::vector<int>> as(ws), at(ws);   // words of the sums of the two kernels
+        for (int i = 0; i < ws; ++i) {
+          const int l = perm[w0 + i];
+          for (int t = he.ptr[l]; t < he.ptr[l + 1]; ++t) {
+            as[i].push_back(pair[t]);
+            if (kj_ok) at[i].push_back(he.k[t] * wts + he.j[t]);
+          }
         }
+        const WarpSchedule ss = schedule_warp(as);
+        const WarpSchedule st = kj_ok ? schedule_warp(at) : ss;
+        for (size_t c = 0; c < ss.size(); ++c)
+          for (int i = 0; i < ws; ++i) {
+            const int b = he.ptr[perm[w0 + i]], qs = ss[c][i], qt = st[c][i];
+            const size_t o = (size_t)tb[w0 + i] + 32 * c;   // padding stays the zero word
+            if (qs >= 0) packed[o] = ((unsigned)as[i][qs] << 12) | (unsigned)cls.at(he.c[b + qs]) << 2;
+            if (qt >= 0 && kj_ok) pkj[o] = ((unsigned)cls.at(he.c[b + qt]) << 24) | (unsigned)at[i][qt];
+          }
       }
       if (E.nout < 65536) {
         // per slot: its first word and (output << 16 | couplings of the
@@ -183,6 +265,7 @@ static void free_edges(EdgeList& E) {
   cudaFree(E.sdesc);
   cudaFree(E.ctab);
   cudaFree(E.ctab32);
+  cudaFree(E.pkj);
   cudaFree(E.pk);
   cudaFree(E.pj);
   cudaFree(E.pair);

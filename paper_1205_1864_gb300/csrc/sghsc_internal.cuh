@@ -44,6 +44,11 @@ enum : int {
   ST_OUTER_BREAKDOWN = 4,
 };
 
+// Staged layout of the double-float products (dfprod.cu): floats per term row
+// and per input column.
+constexpr int DF_VS = 20;
+constexpr int DF_XS = 12;
+
 // Sparse G coupling in gather form: for output chaos column l (local index in
 // the output range), edges ptr[l]..ptr[l+1] with KL index k (1..M), input
 // column j (local index in the input range) and coefficient c = (G_k)_{lj}.
@@ -64,19 +69,25 @@ struct EdgeList {
   int* pk = nullptr;
   int* pj = nullptr;
   int* pair = nullptr;
-  // Compact coupling table: pair << 8 | class per coupling, the coefficient of
-  // class c in ctab[c] (df64). The coefficients of the linear KL expansion take
+  // Compact coupling table: sum position and class per coupling, the coefficient
+  // of class c in ctab[c] (df64). The coefficients of the linear KL expansion take
   // one value per 1-D degree, so a few classes cover them; ncls = 0 when the
   // table does not compress (more than 256 distinct coefficients).
-  // couplings packed (pair << 8 | coefficient class), slot-transposed: the
-  // c-th coupling of output slot s (perm order) at ctr[tb(s) + 32 c], so the
-  // lanes of a warp (32 consecutive slots) read consecutive words; tb(s) is
-  // in the slot's descriptor (sdesc)
+  // couplings packed (byte offset of the term sum << 10 | byte offset of the
+  // coefficient class), slot-transposed: the
+  // word of step c of output slot s (perm order) at ctr[tb(s) + 32 c], so the
+  // lanes of a warp (32 consecutive slots) read consecutive words; tb(s) is in
+  // the slot's descriptor (sdesc). The order of an output's couplings over the
+  // steps is chosen per warp so that their sums lie in different shared-memory
+  // banks.
   unsigned* ctr = nullptr;
-  // the same positions packed as class << 24 | (k rows32_stride(nin) + j)
-  // (below 2^24)
+  // the pairs as staged offsets of the double-float products, k DF_VS << 16 | j DF_XS
+  // (null when one does not fit 16 bits)
+  unsigned* pkj = nullptr;
+  // the same for the FP32 row kernel: class << 24 | (k rows32_stride(nin) + j)
+  // (below 2^24), in an order of its own
   unsigned* ckj = nullptr;
-  int2* sdesc = nullptr;     // per slot: tb(s), output << 16 | couplings
+  int2* sdesc = nullptr;     // per slot: tb(s), output << 16 | steps of its warp
   void* ctab = nullptr;      // df64
   float* ctab32 = nullptr;   // the same coefficients in FP32
   int ncls = 0;

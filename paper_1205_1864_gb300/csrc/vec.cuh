@@ -60,8 +60,9 @@ __device__ __forceinline__ void tree_sum2(double* r0, double* r1) {
 // Fixed-order block sum of (v0, v1) to part[blockIdx]; returns true in the last
 // block, whose threads then hold the totals (t0, t1) over all blocks (summed in
 // block order). blockDim <= 1024.
-__device__ __forceinline__ bool outer_reduce_last(double v0, double v1, const OuterArgs& a, double& t0, double& t1) {
-  __shared__ double r0[1024], r1[1024];
+// r0, r1: shared memory for blockDim doubles each.
+__device__ __forceinline__ bool outer_reduce_last(double v0, double v1, const OuterArgs& a, double& t0, double& t1,
+                                                  double* r0, double* r1) {
   __shared__ bool last;
   r0[threadIdx.x] = v0;
   r1[threadIdx.x] = v1;
@@ -89,6 +90,10 @@ __device__ __forceinline__ bool outer_reduce_last(double v0, double v1, const Ou
   t1 = r1[0];
   if (threadIdx.x == 0) a.ctl->ticket = 0;
   return true;
+}
+__device__ __forceinline__ bool outer_reduce_last(double v0, double v1, const OuterArgs& a, double& t0, double& t1) {
+  __shared__ double r0[1024], r1[1024];
+  return outer_reduce_last(v0, v1, a, t0, t1, r0, r1);
 }
 
 
