@@ -137,10 +137,19 @@ static Shape fit(const sg_problem* h, Shape s, K kern) {
   return s;
 }
 
+// Width of a batch of w columns in the workspace: whole 16-byte pieces, and
+// from 97 FP32 columns on whole 128-byte lines, so that a strip's part of a
+// node is one line and not parts of two (as long as n times the width stays
+// within 32 bits).
 template <typename T>
-static int padded_width(int w) {
+static int vector_width(int w) {
   constexpr int N = 16 / (int)sizeof(T);
   return (w + N - 1) / N * N;
+}
+template <typename T>
+static int padded_width(int w, int n) {
+  const int lines = (w + 31) / 32 * 32;
+  return sizeof(T) == 4 && w > 96 && (long long)n * lines < (1LL << 31) ? lines : vector_width<T>(w);
 }
 
 enum { FIN_INIT = 0, FIN_RHO = 1, FIN_ALPHA = 2, FIN_CONV = 3 };
@@ -1640,7 +1649,63 @@ __global__ void __launch_bounds__(pipe::NT, 1)
   }
 }
 
+#include "mg_fused.cuh"
+
 // ------------------------------------------------------------ host side ---
+
+// The V-cycle's work on grid G in two passes (mg_fused.cuh): FP32, two sweeps
+// each way. Strips of 8 columns for narrow batches, which are bound by the
+// launches and a block's row steps (up to 24 columns; 40 on grids as large as
+// 511 x 511, whose rows keep every SM busy), of 32 columns for batches that
+// stream from memory (n x w from 4.5 million on). Between the two the
+// kernel-per-sweep forms fill the chip better. One V-cycle, two-pass against
+// kernel-per-sweep: 127 x 127 x 4 columns 97 against 189 us, x 330 222
+// against 251, x 126 (not taken) 159 against 135; 255 x 255 x 20 154 against
+// 175, x 330 478 against 679; 511 x 511 x 36 323 against 377, x 715 2761
+// against 4433 us.
+static bool fused_narrow(const GridLevel& G, int wp) { return wp <= (G.n >= 200000 ? 40 : 24); }
+template <typename T>
+static bool use_fused(const sg_problem* h, const GridLevel& G, const GridLevel& C, int wp, const sg_prec_opts& o) {
+  return sizeof(T) == 4 && o.nu == 2 && !h->pipe_off && G.nx == 2 * C.nx + 1 && G.ny == 2 * C.ny + 1 &&
+         (fused_narrow(G, wp) || (long long)G.n * wp >= 4500000);
+}
+
+// Blocks of a pass over tot strip rows: what is resident, but at least four
+// rows each (a run's first and last steps form no output).
+template <typename K>
+static int fused_grid(const sg_problem* h, K kern, int threads, size_t smem, long long tot, int* grid) {
+  SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+  *grid = (int)std::min<long long>((tot + 3) / 4, (long long)h->num_sms * std::max(1, std::min(per_sm, 8)));
+  return SG_OK;
+}
+
+template <int PG>
+static int launch_down(sg_problem* h, const GridLevel& G, const GridLevel& C, int wp, const float* b, float* bc,
+                       float om, const int* done, cudaStream_t s) {
+  auto kern = k_mg_down<PG>;
+  const size_t smem = mg_smem_bytes<PG, false>();
+  int grid = 0;
+  SG_TRY(fused_grid(h, kern, mg::LX * PG, smem,
+                    (long long)ceil_div(wp, 4 * PG) * ceil_div(C.nx, mg::OUT / 2) * C.ny, &grid));
+  { kern<<<grid, mg::LX * PG, smem, s>>>(G.nx, G.ny, C.nx, C.ny, wp, G.st12, b, bc, om, done); ::sghsc::note_launch(); }
+  SG_CHECK_LAUNCH();
+  return SG_OK;
+}
+
+template <int PG, bool DOT>
+static int launch_up(sg_problem* h, const GridLevel& G, const GridLevel& C, int wp, const float* b, const float* xc,
+                     float* out, float om, const FinArgs& f, cudaStream_t s) {
+  auto kern = k_mg_up<PG, DOT>;
+  const size_t smem = mg_smem_bytes<PG, true>();
+  int grid = 0;
+  SG_TRY(fused_grid(h, kern, mg::LX * PG, smem, (long long)ceil_div(wp, 4 * PG) * ceil_div(G.nx, mg::OUT) * G.ny,
+                    &grid));
+  { kern<<<grid, mg::LX * PG, smem, s>>>(G.nx, G.ny, C.nx, C.ny, wp, G.st12, b, xc, out, om, f); ::sghsc::note_launch(); }
+  SG_CHECK_LAUNCH();
+  return SG_OK;
+}
 
 // Row-pipelined sweeps (k_pipe: the Jacobi sweeps and the two sweeps from
 // zero) on grids of at least pipe::MIN_NODES nodes, FP32 batches of 64 columns
@@ -1697,7 +1762,7 @@ int ensure_inner_work(sg_problem* h, int dtype, int wcap) {
     return SG_ERR_UNSUPPORTED;
   }
   InnerWork& iw = dtype == SG_F64 ? h->iw64 : h->iw32;
-  wcap = (wcap + 3) / 4 * 4;   // room for the padded width of either precision
+  wcap = std::max((wcap + 3) / 4 * 4, padded_width<float>(wcap, h->grids[0].n));   // room for either precision
   if (iw.wcap >= wcap) return SG_OK;
   if (h->capturing) {
     set_error("inner solve: workspace must be allocated before graph capture");
@@ -1901,6 +1966,22 @@ static int vcycle(sg_problem* h, InnerWork& iw, int g, const T* b, T* x, T* xt, 
   const GridLevel& C = h->grids[g + 1];
   const T* st = sizeof(T) == 8 ? (const T*)G.st64 : (const T*)G.st32;
   const T* dinv = sizeof(T) == 8 ? (const T*)G.dinv64 : (const T*)G.dinv32;
+  if constexpr (sizeof(T) == 4) {
+    if (use_fused<T>(h, G, C, wp, o)) {
+      float* bc = (float*)iw.cb[g + 1];
+      const float* xc = nullptr;
+      const bool wide = !fused_narrow(G, wp);
+      if (wide) SG_TRY(launch_down<8>(h, G, C, wp, b, bc, om, iw.done, s));
+      else SG_TRY(launch_down<2>(h, G, C, wp, b, bc, om, iw.done, s));
+      SG_TRY(vcycle<T>(h, iw, g + 1, bc, (T*)iw.cx[g + 1], (T*)iw.cxt[g + 1], wp, o, s, nullptr, &xc));
+      if (fdot && wide) SG_TRY((launch_up<8, true>(h, G, C, wp, b, xc, x, om, *fdot, s)));
+      else if (fdot) SG_TRY((launch_up<2, true>(h, G, C, wp, b, xc, x, om, *fdot, s)));
+      else if (wide) SG_TRY((launch_up<8, false>(h, G, C, wp, b, xc, x, om, fz, s)));
+      else SG_TRY((launch_up<2, false>(h, G, C, wp, b, xc, x, om, fz, s)));
+      *out = x;
+      return SG_OK;
+    }
+  }
   const Shape sh = make_shape(h, G.n, ng);
   const Shape shd = make_shape(h, G.n, ng, 1);   // kernels that end in a reduction
   T* cur = x;
@@ -1960,7 +2041,7 @@ static int inner_solve_t(sg_problem* h, const void* src, int ld_src, int src_t, 
   constexpr int N = VW<T>::N;
   InnerWork& iw = sizeof(T) == 8 ? h->iw64 : h->iw32;
   const GridLevel& G = h->grids[0];
-  const int wp = padded_width<T>(w), ng = wp / N;
+  const int wp = padded_width<T>(w, G.n), ng = wp / N;
   const Shape sh = make_shape(h, G.n, ng, 1);    // gather / matvec / update end in reductions
   const Shape shs = make_shape(h, G.n, ng);
   T* x = (T*)iw.x;
@@ -2020,11 +2101,10 @@ int inner_solve(sg_problem* h, int dtype, const void* src, int ld_src, int src_t
 // packed into the padded workspace, the cycle runs there, the result is
 // unpacked into X.
 template <typename T>
-static int vcycle_packed(sg_problem* h, InnerWork& iw, const T* B, T* bpad, T* X, int w, const sg_prec_opts& o,
-                         cudaStream_t s) {
+static int vcycle_packed(sg_problem* h, InnerWork& iw, const T* B, T* bpad, T* X, int w, int wp,
+                         const sg_prec_opts& o, cudaStream_t s) {
   constexpr int N = VW<T>::N;
   const GridLevel& G = h->grids[0];
-  const int wp = padded_width<T>(w);
   const Shape sh = make_shape(h, G.n, wp / N);
   { k_pack<T, T><<<sh.grid, sh.bdim, 0, s>>>(G.n, w, wp, sh.k, B, w, bpad); ::sghsc::note_launch(); }
   const T* res = nullptr;
@@ -2043,7 +2123,7 @@ static int m0_apply_t(sg_problem* h, const T* src, int lds, T* dst, int ldd, int
   constexpr int N = VW<T>::N;
   InnerWork& iw = sizeof(T) == 8 ? h->iw64 : h->iw32;
   const GridLevel& G = h->grids[0];
-  const int wp = padded_width<T>(w);
+  const int wp = padded_width<T>(w, G.n);
   const Shape sh = make_shape(h, G.n, wp / N);
   { k_clear_done<<<1, 1024, 0, s>>>(iw.wcap, iw.done); ::sghsc::note_launch(); }
   { k_pack<T, T><<<sh.grid, sh.bdim, 0, s>>>(G.n, w, wp, sh.k, src, lds, (T*)iw.r); ::sghsc::note_launch(); }
@@ -2071,8 +2151,11 @@ int inner_vcycle(sg_problem* h, int dtype, const void* B, void* X, int w, const 
   SG_TRY(ensure_inner_work(h, dtype, std::max(w, h->wmax)));
   InnerWork& iw = dtype == SG_F64 ? h->iw64 : h->iw32;
   { k_clear_done<<<1, 1024, 0, s>>>(iw.wcap, iw.done); ::sghsc::note_launch(); }
-  if (dtype == SG_F64) return vcycle_packed<double>(h, iw, (const double*)B, (double*)iw.r, (double*)X, w, o, s);
-  return vcycle_packed<float>(h, iw, (const float*)B, (float*)iw.r, (float*)X, w, o, s);
+  const int n = h->grids[0].n;
+  if (dtype == SG_F64)
+    return vcycle_packed<double>(h, iw, (const double*)B, (double*)iw.r, (double*)X, w, padded_width<double>(w, n), o,
+                                 s);
+  return vcycle_packed<float>(h, iw, (const float*)B, (float*)iw.r, (float*)X, w, padded_width<float>(w, n), o, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -2141,7 +2224,7 @@ int vcycle_static(sg_problem* h, int dtype, const void* B, void* X, int w, const
     return SG_ERR_UNSUPPORTED;
   }
   const size_t es = dtype == SG_F64 ? 8 : 4;
-  const int wp = dtype == SG_F64 ? padded_width<double>(w) : padded_width<float>(w);
+  const int wp = dtype == SG_F64 ? vector_width<double>(w) : vector_width<float>(w);
   const size_t need = static_vcycle_bytes(h, wp, es);
   if (need > STATIC_SCRATCH_BYTES) {
     set_error("sg_vcycle_apply_static: %d columns of %d nodes need %zu bytes of scratch, above the fixed %zu",
@@ -2177,8 +2260,8 @@ int vcycle_static(sg_problem* h, int dtype, const void* B, void* X, int w, const
   }
   // the kernels skip columns whose done flag is set: start from all zero
   SG_TRY_CUDA(cudaMemsetAsync(sw.done, 0, (size_t)wp * sizeof(int), s));
-  if (dtype == SG_F64) return vcycle_packed<double>(h, sw, (const double*)B, (double*)sw.r, (double*)X, w, o, s);
-  return vcycle_packed<float>(h, sw, (const float*)B, (float*)sw.r, (float*)X, w, o, s);
+  if (dtype == SG_F64) return vcycle_packed<double>(h, sw, (const double*)B, (double*)sw.r, (double*)X, w, wp, o, s);
+  return vcycle_packed<float>(h, sw, (const float*)B, (float*)sw.r, (float*)X, w, wp, o, s);
 }
 
 }  // namespace sghsc

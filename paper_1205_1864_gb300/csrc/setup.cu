@@ -60,6 +60,15 @@ static int upload(T** dst, const T* src, size_t count) {
   return SG_OK;
 }
 
+// FP32 stencils [n][9] and inverse diagonals into 48-byte records (GridLevel::st12)
+__global__ void k_pack_stencil(int n, const float* __restrict__ st, const float* __restrict__ dinv,
+                               float* __restrict__ st12) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * 12; i += gridDim.x * blockDim.x) {
+    const int node = i / 12, e = i - node * 12, c = e & 3;
+    st12[i] = c < 3 ? st[node * 9 + e / 4 * 3 + c] : (e == 11 ? dinv[node] : 0.f);
+  }
+}
+
 struct HostEdges {
   std::vector<int> ptr{0}, k, j;
   std::vector<double> c;
@@ -68,62 +77,56 @@ struct HostEdges {
 // The order in which the 32 output slots of a warp take their couplings, so
 // that the words a warp reads together lie in different shared-memory banks
 // (in list order a step's reads met up to eight deep in one bank). addr[s]:
-// word address of each coupling of slot s; row c of the result holds, per slot,
-// the index of the coupling taken at step c, or -1 (padding). As many rows as
+// word address of each coupling of slot s; entry c * 32 + s of the result is
+// the coupling that slot s takes at step c, or -1 (padding). As many steps as
 // the longest list. Greedy: at each step the slots with most left choose
 // first, the address that shares its bank with the fewest others; a slot with
 // steps to spare waits rather than collide.
-using WarpSchedule = std::vector<std::vector<int>>;
-static WarpSchedule schedule_warp(const std::vector<std::vector<int>>& addr) {
-  WarpSchedule w;
-  const int n = (int)addr.size();
-  size_t rows = 0;
-  std::vector<std::vector<int>> left(n);
-  std::vector<int> demand(32, 0);
+static std::vector<int> schedule_warp(const std::vector<int>* addr, int n) {
+  int rows = 0;
+  std::vector<int> left[32];
+  int demand[32] = {0}, order[32];
   for (int s = 0; s < n; ++s) {
-    rows = std::max(rows, addr[s].size());
+    rows = std::max(rows, (int)addr[s].size());
+    order[s] = s;
     for (int i = 0; i < (int)addr[s].size(); ++i) {
       left[s].push_back(i);
       ++demand[addr[s][i] & 31];
     }
   }
-  std::vector<int> order(n);
+  std::vector<int> take((size_t)rows * 32, -1);
   if (rows > 64) {   // the dense couplings of a gPC coefficient: list order (the search is quadratic)
-    for (size_t r = 0; r < rows; ++r) {
-      std::vector<int> take(n, -1);
-      for (int s = 0; s < n; ++s)
-        if (r < addr[s].size()) take[s] = (int)r;
-      w.push_back(take);
-    }
-    return w;
+    for (int s = 0; s < n; ++s)
+      for (int r = 0; r < (int)addr[s].size(); ++r) take[(size_t)r * 32 + s] = r;
+    return take;
   }
-  for (size_t r = 0; r < rows; ++r) {
-    std::vector<int> take(n, -1);
-    std::vector<std::vector<int>> bank(32);   // distinct addresses read so far
-    for (int s = 0; s < n; ++s) order[s] = s;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return left[a].size() > left[b].size(); });
-    for (int s : order) {
+  for (int r = 0; r < rows; ++r) {
+    int cnt[32] = {0}, seen[32][32];   // distinct addresses read so far, by bank
+    auto in = [&](int a) {
+      for (int i = 0; i < cnt[a & 31]; ++i)
+        if (seen[a & 31][i] == a) return true;
+      return false;
+    };
+    std::stable_sort(order, order + n, [&](int a, int b) { return left[a].size() > left[b].size(); });
+    for (int o = 0; o < n; ++o) {
+      const int s = order[o];
       int best = -1, cost = 0;
       for (int q = 0; q < (int)left[s].size(); ++q) {
-        const int a = addr[s][left[s][q]];
-        const auto& B = bank[a & 31];
-        const int c = std::count(B.begin(), B.end(), a) ? 0 : (int)B.size();
+        const int a = addr[s][left[s][q]], c = in(a) ? 0 : cnt[a & 31];
         if (best < 0 || c < cost || (c == cost && demand[a & 31] > demand[addr[s][left[s][best]] & 31])) {
           best = q;
           cost = c;
         }
       }
-      if (best < 0 || (cost > 0 && left[s].size() < rows - r)) continue;
+      if (best < 0 || (cost > 0 && (int)left[s].size() < rows - r)) continue;
       const int a = addr[s][left[s][best]];
-      auto& B = bank[a & 31];
-      if (!std::count(B.begin(), B.end(), a)) B.push_back(a);
+      if (!in(a)) seen[a & 31][cnt[a & 31]++] = a;
       --demand[a & 31];
-      take[s] = left[s][best];
+      take[(size_t)r * 32 + s] = left[s][best];
       left[s].erase(left[s].begin() + best);
     }
-    w.push_back(take);
   }
-  return w;
+  return take;
 }
 
 static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 = 0, int nin = 0) {
@@ -202,9 +205,11 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 
       const int wts = rows32_stride(nin);   // the row stride of the FP32 row kernel's term sums
       for (int t = 0; t < E.nedges; ++t) kj_ok = kj_ok && (long long)he.k[t] * wts + he.j[t] < (1 << 24);
       if (kj_ok) pkj.assign(packed.size(), 0u);
+      std::vector<unsigned> cof(E.nedges);
+      for (int t = 0; t < E.nedges; ++t) cof[t] = (unsigned)cls.at(he.c[t]);
       for (int w0 = 0; w0 < E.nout; w0 += 32) {
         const int ws = std::min(32, E.nout - w0);
-        std::vector<std::vector<int>> as(ws), at(ws);   // words of the sums of the two kernels
+        std::vector<int> as[32], at[32];   // words of the sums of the two kernels
         for (int i = 0; i < ws; ++i) {
           const int l = perm[w0 + i];
           for (int t = he.ptr[l]; t < he.ptr[l + 1]; ++t) {
@@ -212,14 +217,14 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 
             if (kj_ok) at[i].push_back(he.k[t] * wts + he.j[t]);
           }
         }
-        const WarpSchedule ss = schedule_warp(as);
-        const WarpSchedule st = kj_ok ? schedule_warp(at) : ss;
-        for (size_t c = 0; c < ss.size(); ++c)
+        const std::vector<int> ss = schedule_warp(as, ws);
+        const std::vector<int> st = kj_ok ? schedule_warp(at, ws) : ss;
+        for (size_t c = 0; c < ss.size() / 32; ++c)
           for (int i = 0; i < ws; ++i) {
-            const int b = he.ptr[perm[w0 + i]], qs = ss[c][i], qt = st[c][i];
+            const int b = he.ptr[perm[w0 + i]], qs = ss[c * 32 + i], qt = st[c * 32 + i];
             const size_t o = (size_t)tb[w0 + i] + 32 * c;   // padding stays the zero word
-            if (qs >= 0) packed[o] = ((unsigned)as[i][qs] << 12) | (unsigned)cls.at(he.c[b + qs]) << 2;
-            if (qt >= 0 && kj_ok) pkj[o] = ((unsigned)cls.at(he.c[b + qt]) << 24) | (unsigned)at[i][qt];
+            if (qs >= 0) packed[o] = ((unsigned)as[i][qs] << 12) | cof[b + qs] << 2;
+            if (qt >= 0 && kj_ok) pkj[o] = cof[b + qt] << 24 | (unsigned)at[i][qt];
           }
       }
       if (E.nout < 65536) {
@@ -389,6 +394,9 @@ static int upload_grid(GridLevel& g, const std::vector<double>& st) {
   SG_TRY(upload(&g.st32, st32.data(), st32.size()));
   SG_TRY(upload(&g.dinv64, dinv.data(), dinv.size()));
   SG_TRY(upload(&g.dinv32, dinv32.data(), dinv32.size()));
+  SG_TRY_CUDA(cudaMalloc((void**)&g.st12, dinv32.size() * 12 * sizeof(float)));
+  { k_pack_stencil<<<std::min(((int)dinv32.size() * 12 + 255) / 256, 4096), 256>>>((int)dinv32.size(), g.st32, g.dinv32, g.st12); ::sghsc::note_launch(); }
+  SG_CHECK_LAUNCH();
   return SG_OK;
 }
 
@@ -617,14 +625,17 @@ __global__ void k_scale_vals(long long count, int M1, const double* __restrict__
 
 // multigrid stencils of s * A_0: st = s * base, dinv = 1 / (s * base_centre)
 __global__ void k_scale_grid(int n, const double* __restrict__ base, double s, double* __restrict__ st64,
-                             float* __restrict__ st32, double* __restrict__ dinv64, float* __restrict__ dinv32) {
+                             float* __restrict__ st32, double* __restrict__ dinv64, float* __restrict__ dinv32,
+                             float* __restrict__ st12) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * 9; i += gridDim.x * blockDim.x) {
     const double v = s * base[i];
     st64[i] = v;
     st32[i] = (float)v;
+    st12[i / 9 * 12 + i % 9 / 3 * 4 + i % 3] = (float)v;
     if (i % 9 == 4) {
       dinv64[i / 9] = 1.0 / v;
       dinv32[i / 9] = (float)(1.0 / v);
+      st12[i / 9 * 12 + 11] = (float)(1.0 / v);
     }
   }
 }
@@ -656,7 +667,7 @@ int sg_set_scales(sg_problem* h, const double* scale) {
   const long long count = (long long)h->nnz * h->nterm;
   { k_scale_vals<<<(int)std::min<long long>((count + 255) / 256, 4096), 256>>>(count, h->nterm, h->vals_base, h->scales_dev, h->vals64, h->vals32, (df64*)h->vals_df); ::sghsc::note_launch(); }
   for (auto& g : h->grids)
-    { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g.n, g.st_base, scale[0], g.st64, g.st32, g.dinv64, g.dinv32); ::sghsc::note_launch(); }
+    { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g.n, g.st_base, scale[0], g.st64, g.st32, g.dinv64, g.dinv32, g.st12); ::sghsc::note_launch(); }
   SG_TRY_CUDA(cudaGetLastError());
   SG_TRY_CUDA(cudaDeviceSynchronize());
   return SG_OK;
@@ -754,7 +765,7 @@ void sg_destroy(sg_problem* h) {
   free_edges(h->sub);
   for (auto& e : h->dlev) free_edges(e);
   for (auto& g : h->grids) {
-    cudaFree(g.st_base); cudaFree(g.st64); cudaFree(g.st32); cudaFree(g.dinv64); cudaFree(g.dinv32);
+    cudaFree(g.st_base); cudaFree(g.st64); cudaFree(g.st32); cudaFree(g.dinv64); cudaFree(g.dinv32); cudaFree(g.st12);
   }
   if (h->cap[0]) cudaDeviceSynchronize();
   clear_graphs(h);

@@ -103,6 +103,9 @@ struct GridLevel {
   float* st32 = nullptr;
   double* dinv64 = nullptr;
   float* dinv32 = nullptr;
+  // FP32 stencil and inverse diagonal of a node in 48 bytes, three 16-byte
+  // pieces: the row above, the own row, the row below with dinv in its last slot
+  float* st12 = nullptr;
 };
 
 // Device control block of one batched inner solve.
