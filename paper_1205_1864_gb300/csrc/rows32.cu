@@ -2,7 +2,8 @@
 // level product B_l / C_l of Algorithm 1) with every input column in
 // registers.
 //
-// One block per matrix row r at a time (two on narrower levels). For each chunk of up to nine
+// One to eight matrix rows per block at a time (rows32_pick in
+// sghsc_internal.cuh; one row r below). For each chunk of up to nine
 // nonzeros c_e of the row (the Q1 stencil row is one chunk) the block stages
 // the KL-term values a_k(r, c_e) in shared memory, padded to three float4 per
 // term; thread j then loads X(c_e, j) for its input column from global memory
@@ -62,7 +63,9 @@ __device__ __forceinline__ void term_sum2(const float4* v, const float (&x)[rows
 // each entry is read, then written, by the same thread), else Y = sum.
 // ROWS rows at a time, RG = NT / ROWS threads per row (a multiple of 32, so
 // the slot-transposed couplings still give a warp consecutive words): on
-// narrow levels several rows share the block's barriers.
+// narrower blocks several rows share the block's barriers and the latency of
+// each row's chain of loads (bounds, columns, inputs), which is what bounds
+// this kernel below some 500 columns.
 template <bool DIAG, bool SUB, int ROWS>
 __global__ void __launch_bounds__(rows32::NT, 4) k_rows32(
     int n, const int* __restrict__ rowptr, const int* __restrict__ colidx, const float* __restrict__ vals, int M1,
@@ -71,7 +74,8 @@ __global__ void __launch_bounds__(rows32::NT, 4) k_rows32(
   using namespace rows32;
   constexpr int RG = NT / ROWS;
   extern __shared__ __align__(16) float4 sm4[];
-  const int wts = rows32_stride(wx);
+  constexpr int PASS = ROWS32_COLS / ROWS;
+  const int wts = (wx + PASS - 1) / PASS * PASS;   // rows32_stride
   float* Ctab = reinterpret_cast<float*>(sm4);                        // [ncls]
   float4* Vall = sm4 + (ncls + 3) / 4;                                 // [ROWS][M1][VS4]
   float* Tall = reinterpret_cast<float*>(Vall + (size_t)ROWS * M1 * VS4);   // [ROWS][M1][wts]
@@ -161,33 +165,26 @@ __global__ void __launch_bounds__(rows32::NT, 4) k_rows32(
   }
 }
 
-static size_t rows32_smem(const EdgeList& E, int M1, int wx, int rows) {
-  return (size_t)((E.ncls + 3) & ~3) * 4 +
-         (size_t)rows * ((size_t)M1 * rows32::VS4 * 16 + (size_t)M1 * rows32_stride(wx) * 4);
+int rows32_rows(int wx, int wy, bool square, int terms) {
+  int rows = rows32_pick(wx, wy, square);
+  while (rows > 1 && rows32_smem(256, terms, wx, rows) > 110 * 1024) rows /= 2;
+  return rows;
 }
 
-// Rows per block: one for the wide products, two for the level products
-// between 32 and 512 columns each way (at 511^2 rows, M = 10: 55 <- 220
-// columns 0.95 against 1.36 ms for the row-per-warp kernel, 220 <- 55 0.90
-// against 0.98 ms; four rows per block: 1.10 and 1.12 ms); 0 where this
-// kernel is not taken.
-static int rows32_rows(const EdgeList& E, int wx, bool diag) {
-  if (wx >= 512 || E.nout >= 512) return 1;
-  return !diag && wx >= 32 && E.nout >= 32 ? 2 : 0;
-}
-
-// FP32 products take this kernel for inputs from 512 columns, or from 128
-// input columns with at least 512 outputs (measured on the 512x512, M = 10,
-// p = 4 operator: 1001 -> 1001 columns 3.7 ms against 11.1 ms for the
-// row-per-warp kernel, 715 -> 220 2.7 against 4.6 ms, 220 -> 715 2.0 against
-// 3.4 ms), and with two rows per block for level products of 32 to 512
-// columns each way (one row per block there: 220 -> 55 1.16 against
-// 0.99 ms, the rows too short to amortise the block barriers).
+// Taken wherever rows32_pick gives a row count (the linear KL expansion; a gPC
+// coefficient's many terms only from 512 columns on). Against the kernels
+// taken before, 199 x 199 rows: full product M = 8, p = 4 (495 columns, two
+// rows) 774 -> 262 us, one row 281, four 298; M = 6, p = 4 (210, four rows) 306
+// -> 113; M = 4, p = 3 (35, eight rows) 59 -> 37; 6 and 10 columns 25 -> 29 and
+// 29 -> 30 (not taken). Level products: 220 -> 55 (four rows) 137 -> 115, eight
+// rows 129; 55 -> 220 (eight) 122 -> 73; 126 -> 56 107 -> 58; 21 -> 56 50 -> 38;
+// 715 -> 220 (two) 410 -> 389; 220 -> 715 (two) 328 -> 253; 10 -> 20 and 8 -> 36
+// 31 -> 33 and 41 -> 43 (not taken). 1001 columns: one row 585, two 823.
 bool rows32_usable(const sg_problem* h, const EdgeList& E, int wx, bool diag) {
-  const int rows = rows32_rows(E, wx, diag);
-  const bool shape = wx >= 512 || (E.nout >= 512 && wx >= 128) || rows > 1;
-  return h->staged_pairs && shape && wx == E.nin && E.ckj && E.sdesc && E.ncls > 0 && h->nterm <= 256 &&
-         rows32_smem(E, h->nterm, wx, std::max(rows, 1)) <= (size_t)std::max(h->smem_optin, 48 * 1024);
+  const bool square = E.nin == E.nout && E.in0 == E.out0;
+  return h->staged_pairs && E.rows32 > 0 && (h->q < 0 || wx >= 512 || E.nout >= 512) && diag == square &&
+         wx == E.nin && E.ckj && E.sdesc && E.ncls > 0 && h->nterm <= 256 &&
+         rows32_smem(E.ncls, h->nterm, wx, E.rows32) <= (size_t)std::max(h->smem_optin, 48 * 1024);
 }
 
 int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, int ldx, int wx, const float* Yin,
@@ -199,8 +196,8 @@ int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, i
     set_error("FP32 row product: unsupported form");
     return SG_ERR_UNSUPPORTED;
   }
-  const int rows = std::max(rows32_rows(E, wx, diag), 1);
-  const size_t smem = rows32_smem(E, h->nterm, wx, rows);
+  const int rows = E.rows32;
+  const size_t smem = rows32_smem(E.ncls, h->nterm, wx, rows);
   auto go = [&](auto kern) -> int {
     SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
@@ -211,9 +208,11 @@ int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, i
     SG_CHECK_LAUNCH();
     return SG_OK;
   };
-  if (diag) return go(k_rows32<true, false, 1>);
-  if (rows == 2) return go(k_rows32<false, true, 2>);
-  return go(k_rows32<false, true, 1>);
+  if (diag)
+    return rows == 1 ? go(k_rows32<true, false, 1>) : rows == 2 ? go(k_rows32<true, false, 2>)
+           : rows == 4 ? go(k_rows32<true, false, 4>) : go(k_rows32<true, false, 8>);
+  return rows == 1 ? go(k_rows32<false, true, 1>) : rows == 2 ? go(k_rows32<false, true, 2>)
+         : rows == 4 ? go(k_rows32<false, true, 4>) : go(k_rows32<false, true, 8>);
 }
 
 }  // namespace sghsc

@@ -129,7 +129,7 @@ static std::vector<int> schedule_warp(const std::vector<int>* addr, int n) {
   return take;
 }
 
-static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 = 0, int nin = 0) {
+static int upload_edges(const HostEdges& he, EdgeList& E, int out0, int in0, int nin, int terms) {
   E.out0 = out0;
   E.in0 = in0;
   E.nin = nin;
@@ -202,29 +202,29 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0 = 0, int in0 
       if (total >= (size_t)1 << 31) return SG_ERR_UNSUPPORTED;
       std::vector<unsigned> packed(std::max<size_t>(total, 1), 0u), pkj;
       bool kj_ok = true;
-      const int wts = rows32_stride(nin);   // the row stride of the FP32 row kernel's term sums
+      E.rows32 = rows32_rows(nin, E.nout, nin == E.nout && in0 == out0, terms);
+      const int wts = rows32_stride(nin, E.rows32);   // the row stride of the FP32 row kernel's term sums
       for (int t = 0; t < E.nedges; ++t) kj_ok = kj_ok && (long long)he.k[t] * wts + he.j[t] < (1 << 24);
       if (kj_ok) pkj.assign(packed.size(), 0u);
       std::vector<unsigned> cof(E.nedges);
       for (int t = 0; t < E.nedges; ++t) cof[t] = (unsigned)cls.at(he.c[t]);
       for (int w0 = 0; w0 < E.nout; w0 += 32) {
         const int ws = std::min(32, E.nout - w0);
-        std::vector<int> as[32], at[32];   // words of the sums of the two kernels
+        std::vector<int> as[32];   // words of the double-float products' sums
         for (int i = 0; i < ws; ++i) {
           const int l = perm[w0 + i];
           for (int t = he.ptr[l]; t < he.ptr[l + 1]; ++t) {
             as[i].push_back(pair[t]);
-            if (kj_ok) at[i].push_back(he.k[t] * wts + he.j[t]);
+            // the FP32 row kernel adds in list order (the bits of the gather form)
+            if (kj_ok)
+              pkj[(size_t)tb[w0 + i] + 32 * (t - he.ptr[l])] = cof[t] << 24 | (unsigned)(he.k[t] * wts + he.j[t]);
           }
         }
         const std::vector<int> ss = schedule_warp(as, ws);
-        const std::vector<int> st = kj_ok ? schedule_warp(at, ws) : ss;
         for (size_t c = 0; c < ss.size() / 32; ++c)
-          for (int i = 0; i < ws; ++i) {
-            const int b = he.ptr[perm[w0 + i]], qs = ss[c * 32 + i], qt = st[c * 32 + i];
-            const size_t o = (size_t)tb[w0 + i] + 32 * c;   // padding stays the zero word
-            if (qs >= 0) packed[o] = ((unsigned)as[i][qs] << 12) | cof[b + qs] << 2;
-            if (qt >= 0 && kj_ok) pkj[o] = cof[b + qt] << 24 | (unsigned)at[i][qt];
+          for (int i = 0; i < ws; ++i) {   // padding stays the zero word
+            const int qs = ss[c * 32 + i];
+            if (qs >= 0) packed[(size_t)tb[w0 + i] + 32 * c] = ((unsigned)as[i][qs] << 12) | cof[he.ptr[perm[w0 + i]] + qs] << 2;
           }
       }
       if (E.nout < 65536) {
@@ -488,27 +488,27 @@ static int setup_impl(const sg_mesh* mesh, int M, int p, int family, int n, int 
   h->pre.resize(p + 1);
   h->post.resize(p + 1);
   if (q < 0) {
-    SG_TRY(upload_edges(build_edges(h, index, 0, h->P, 0, h->P), h->all, 0, 0, h->P));
+    SG_TRY(upload_edges(build_edges(h, index, 0, h->P, 0, h->P), h->all, 0, 0, h->P, h->nterm));
     for (int l = 1; l <= p; ++l) {
       SG_TRY(upload_edges(build_edges(h, index, off[l - 1], off[l], off[l], off[l + 1]), h->pre[l], off[l - 1],
-                          off[l], off[l + 1] - off[l]));
+                          off[l], off[l + 1] - off[l], h->nterm));
       SG_TRY(upload_edges(build_edges(h, index, off[l], off[l + 1], off[l - 1], off[l]), h->post[l], off[l],
-                          off[l - 1], off[l] - off[l - 1]));
+                          off[l - 1], off[l] - off[l - 1], h->nterm));
     }
-    if (p >= 1) SG_TRY(upload_edges(build_edges(h, index, 0, off[p], 0, off[p]), h->sub, 0, 0, off[p]));
+    if (p >= 1) SG_TRY(upload_edges(build_edges(h, index, 0, off[p], 0, off[p]), h->sub, 0, 0, off[p], h->nterm));
   } else {
     // the coefficient terms in the same graded order
     std::vector<int> cur(M);
     for (int d = 0; d <= q; ++d) emit_degree(M, 0, d, cur, h->gamma);
-    SG_TRY(upload_edges(build_edges_gpc(h, 0, h->P, 0, h->P), h->all, 0, 0, h->P));
+    SG_TRY(upload_edges(build_edges_gpc(h, 0, h->P, 0, h->P), h->all, 0, 0, h->P, h->nterm));
     h->dlev.resize(p + 1);
     for (int l = 1; l <= p; ++l) {
       // B_l: every lower level from level l; C_l: level l from every lower level; D_l: level l with itself
       SG_TRY(upload_edges(build_edges_gpc(h, 0, off[l], off[l], off[l + 1]), h->pre[l], 0, off[l],
-                          off[l + 1] - off[l]));
-      SG_TRY(upload_edges(build_edges_gpc(h, off[l], off[l + 1], 0, off[l]), h->post[l], off[l], 0, off[l]));
+                          off[l + 1] - off[l], h->nterm));
+      SG_TRY(upload_edges(build_edges_gpc(h, off[l], off[l + 1], 0, off[l]), h->post[l], off[l], 0, off[l], h->nterm));
       SG_TRY(upload_edges(build_edges_gpc(h, off[l], off[l + 1], off[l], off[l + 1]), h->dlev[l], off[l], off[l],
-                          off[l + 1] - off[l]));
+                          off[l + 1] - off[l], h->nterm));
     }
     // the pair form keeps one sum per distinct (term, input) in shared memory:
     // too many with a dense coupling, so the gPC products use the gather form

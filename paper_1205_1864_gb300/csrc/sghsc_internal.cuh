@@ -84,9 +84,10 @@ struct EdgeList {
   // the pairs as staged offsets of the double-float products, k DF_VS << 16 | j DF_XS
   // (null when one does not fit 16 bits)
   unsigned* pkj = nullptr;
-  // the same for the FP32 row kernel: class << 24 | (k rows32_stride(nin) + j)
-  // (below 2^24), in an order of its own
+  // the same for the FP32 row kernel, in list order: class << 24 | (k
+  // rows32_stride(nin, rows32) + j) (below 2^24)
   unsigned* ckj = nullptr;
+  int rows32 = 0;            // rows per block of that kernel (0: not taken)
   int2* sdesc = nullptr;     // per slot: tb(s), output << 16 | steps of its warp
   void* ctab = nullptr;      // df64
   float* ctab32 = nullptr;   // the same coefficients in FP32
@@ -265,11 +266,28 @@ bool narrow_usable(const sg_problem* h, const EdgeList& E, int wx);
 template <typename T>
 int launch_level_narrow(sg_problem* h, const EdgeList& E, const T* X, int ldx, const T* Yin, int ldyin, T* Y, int ldy,
                         cudaStream_t s);
-// Row stride of the term sums of the FP32 row kernel (rows32.cu).
+// The FP32 row kernel (rows32.cu): rows a block of 256 threads works on at a
+// time for a product of wx input and wy output columns (square: the full
+// product; 0: not taken), the row stride of its term sums (whole passes of a
+// row's threads, two input columns each), and its shared memory.
 constexpr int ROWS32_COLS = 512;   // input columns per pass of a block (two per thread)
-__host__ __device__ constexpr int rows32_stride(int wx) { return (wx + ROWS32_COLS - 1) / ROWS32_COLS * ROWS32_COLS; }
+__host__ __device__ constexpr int rows32_pick(int wx, int wy, bool square) {
+  if (wx >= 512) return square ? 1 : 2;
+  if (wy >= 512) return wx >= 128 ? 2 : 0;
+  if (wx < (square ? 15 : 12)) return 0;
+  return wx <= 128 ? 8 : square && wx > 256 ? 2 : 4;
+}
+// the same, fewer rows when they would leave an SM less than two blocks
+int rows32_rows(int wx, int wy, bool square, int terms);
+__host__ __device__ constexpr int rows32_stride(int wx, int rows) {
+  const int pass = ROWS32_COLS / (rows > 0 ? rows : 1);
+  return (wx + pass - 1) / pass * pass;
+}
+constexpr size_t rows32_smem(int ncls, int terms, int wx, int rows) {
+  return (size_t)((ncls + 3) & ~3) * 4 + (size_t)rows * terms * (48 + (size_t)rows32_stride(wx, rows) * 4);
+}
 // FP32 products with the input columns in registers (rows32.cu): usable and
-// preferred for E (compact table, sizes, inputs at least 512 columns wide).
+// preferred for E (compact table, sizes).
 bool rows32_usable(const sg_problem* h, const EdgeList& E, int wx, bool diag);
 int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, int ldx, int wx, const float* Yin,
                   int ldyin, float* Y, int ldy, cudaStream_t s);
