@@ -393,16 +393,16 @@ __device__ __forceinline__ void phase_sync(bool wm) {
   else __syncthreads();
 }
 
-// One V-cycle from the finest grid's b; returns the buffer that holds the
-// result. Every thread of the block calls it.
+// One V-cycle from grid g0's b; returns the buffer that holds the result.
+// Every thread of the block calls it.
 template <typename T>
-__device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu) {
+__device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu, int g0 = 0) {
   const int tid = threadIdx.x, G = L.G;
   auto wmode = [&](int g) { return L.k[g] <= 2 && g > 0; };
   auto vsize = [&](int g) { const int W = (1 << L.k[g]) + 1; return W * W; };
   auto odd = [&](int s) { return (s & 1) != 0; };
   // the iterate of grid g sits in x or y; pre-smoothing makes nu - 1 exchanges
-  for (int g = 0; g < G; ++g) {
+  for (int g = g0; g < G; ++g) {
     const int W = (1 << L.k[g]) + 1, V = vsize(g), k = L.k[g], n = (W - 2) * (W - 2);
     const bool wm = wmode(g);
     const int nt = wm ? 32 : (int)blockDim.x;
@@ -443,7 +443,7 @@ __device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu) {
     }
   }
   T* res = sm + L.vec[G - 1] + vsize(G - 1);
-  for (int g = G - 2; g >= 0; --g) {
+  for (int g = G - 2; g >= g0; --g) {
     const int W = (1 << L.k[g]) + 1, V = vsize(g), k = L.k[g], n = (W - 2) * (W - 2);
     const int Wc = (1 << L.k[g + 1]) + 1;
     const bool wm = wmode(g);
@@ -592,6 +592,230 @@ __global__ void __launch_bounds__(blk::VNT) k_block_vcycle(BlockArgs a, BlockGri
   if (a.iters && tid == 0) a.iters[col] = S.it;
 }
 
+// ------------------------------------------ V-cycle M_0 on 63 x 63, FP32 ---
+
+// One block of 512 threads per column, as k_block_vcycle, but the finest
+// grid's stencils live in registers (72 a thread: they are what a sweep from
+// shared memory would read most of). Thread (y, s) owns the nodes 4 s .. 4 s + 3
+// and 32 + 4 s .. of row y: a row is read as two 16-byte pieces per thread, the
+// neighbours beside them come from the lanes beside it. The coarse grids run
+// in shared memory through block_vcycle. What bounds it: the barriers and the
+// chains between them (a step is 17 us, some 8 of them on the 31 x 31 grid and
+// below). Read node by node, the stencils took 4 us of a solve of two steps;
+// from planes with rows of 64 they are whole lines.
+namespace blk63 {
+constexpr int NT = 512, NX = 63;
+constexpr int W = 72;                 // row stride: node x at 4 + x, zeros around
+constexpr int VEC = (NX + 2) * W;     // a vector with zero rows above and below
+constexpr int OWN = 64 * 64;          // a vector read by its owners only
+constexpr int FLOATS = 3 * VEC + 3 * OWN;
+}  // namespace blk63
+
+struct Own8 {   // a thread's eight nodes
+  float v[8];
+};
+
+__device__ __forceinline__ Own8 own_ld(const float* p) {   // the second piece 32 nodes on
+  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 32);
+  return Own8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+__device__ __forceinline__ void own_st(float* p, const Own8& o) {
+  *reinterpret_cast<float4*>(p) = make_float4(o.v[0], o.v[1], o.v[2], o.v[3]);
+  *reinterpret_cast<float4*>(p + 32) = make_float4(o.v[4], o.v[5], o.v[6], o.v[7]);
+}
+
+// acc + SIGN A v at the thread's nodes; v: its place in the padded vector
+template <int SIGN>
+__device__ __forceinline__ Own8 own_apply(Own8 acc, const float (&c)[8][9], const float* v, int s) {
+#pragma unroll
+  for (int dy = 0; dy < 3; ++dy) {
+    const Own8 q = own_ld(v + (dy - 1) * blk63::W);
+    // the nodes beside the two pieces, from the neighbouring lanes of the row
+    // (0 beyond its ends: the coefficients there are zero)
+    const float l0 = __shfl_sync(0xffffffffu, q.v[3], (s + 7) & 7, 8);
+    const float l1 = __shfl_sync(0xffffffffu, s == 7 ? q.v[3] : q.v[7], (s + 7) & 7, 8);
+    const float r0 = __shfl_sync(0xffffffffu, s == 0 ? q.v[4] : q.v[0], (s + 1) & 7, 8);
+    const float r1 = __shfl_sync(0xffffffffu, q.v[4], (s + 1) & 7, 8);
+    const float w0[6] = {s == 0 ? 0.f : l0, q.v[0], q.v[1], q.v[2], q.v[3], r0};
+    const float w1[6] = {l1, q.v[4], q.v[5], q.v[6], q.v[7], s == 7 ? 0.f : r1};
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc.v[i] = fmaf(SIGN < 0 ? -c[i][dy * 3 + dx] : c[i][dy * 3 + dx], w0[i + dx], acc.v[i]);
+        acc.v[4 + i] = fmaf(SIGN < 0 ? -c[4 + i][dy * 3 + dx] : c[4 + i][dy * 3 + dx], w1[i + dx], acc.v[4 + i]);
+      }
+  }
+  return acc;
+}
+
+__device__ __forceinline__ float own_dot(const Own8& a, const Own8& b) {
+  float s = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s = fmaf(a.v[i], b.v[i], s);
+  return s;
+}
+
+template <typename TS, typename TD>
+__global__ void __launch_bounds__(blk63::NT, 1)
+    k_block_vcycle63(BlockArgs a, BlockGrids L, float om, int nu, const float* __restrict__ planes,
+                     const TS* __restrict__ src, int lds, TD* __restrict__ dst, int ldd) {
+  using namespace blk63;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ float red[NT / 32];
+  __shared__ BlockScalars<float> S;
+  float* const X = reinterpret_cast<float*>(smem_raw);   // X, Y, P: [VEC]; B, D, U: [OWN]
+  float* const Y = X + VEC;
+  float* const P = Y + VEC;
+  float* const sm = X + FLOATS;                           // the coarse grids
+  const int tid = threadIdx.x, col = blockIdx.x, s = tid & 7, y = tid >> 3;
+  const bool act = y < NX;
+  const int at = (min(y, NX - 1) + 1) * W + 4 + 4 * s;    // the thread's place in a padded vector
+  float* const B = P + VEC + y * 64 + 4 * s;              // residual, damped inverse diagonal, solution
+  float* const D = B + OWN;
+  float* const U = D + OWN;
+  for (int i = tid; i < 3 * VEC; i += NT) X[i] = 0.f;
+  for (int g = 1; g < L.G; ++g) {
+    const int Wg = (1 << L.k[g]) + 1, ng = (Wg - 2) * (Wg - 2);
+    for (int i = tid; i < 3 * Wg * Wg; i += NT) sm[L.vec[g] + i] = 0.f;
+    const float* gs = (const float*)L.st[g];
+    const float* gd = (const float*)L.dinv[g];
+    for (int i = tid; i < 9 * ng; i += NT) sm[L.coef[g] + i] = gs[i];
+    for (int i = tid; i < ng; i += NT) sm[L.coef[g] + 9 * ng + i] = g == L.G - 1 ? gd[i] : om * gd[i];
+  }
+  float c[8][9];
+  {
+    Own8 b;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int x = 4 * s + (i & 3) + (i >= 4 ? 32 : 0);
+      b.v[i] = act && x < NX ? widen<float>(src[(size_t)(y * NX + x) * lds + col]) : 0.f;
+    }
+    // the planes' rows are padded with zeros to 64 columns; the last thread row
+    // takes the last grid row's and never publishes what it makes of them
+    const float* pl = planes + min(y, NX - 1) * 64 + 4 * s;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const Own8 q = own_ld(pl + e * NX * 64);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) c[i][e] = act ? q.v[i] : 0.f;
+    }
+    Own8 d = own_ld(pl + 9 * NX * 64);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) d.v[i] = act ? om * d.v[i] : 0.f;
+    own_st(D, d);
+    own_st(B, b);
+    own_st(U, Own8{{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}});
+    block_sum(red, own_dot(b, b), [&](double v) { scal_init(S, v, a); });
+  }
+  while (!S.done) {
+    Own8 cur;
+    {
+      const Own8 b = own_ld(B), d = own_ld(D);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) cur.v[i] = d.v[i] * b.v[i];
+    }
+    float *v = X, *o = Y;
+    if (act) own_st(v + at, cur);
+    __syncthreads();
+    // one more sweep of the iterate in v, its new values in cur
+    auto sweep = [&]() {
+      const Own8 r = own_apply<-1>(own_ld(B), c, v + at, s), d = own_ld(D);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) cur.v[i] = fmaf(d.v[i], r.v[i], cur.v[i]);
+    };
+    auto publish = [&]() {
+      if (act) own_st(o + at, cur);
+      __syncthreads();
+      float* t = v; v = o; o = t;
+    };
+    for (int it = 1; it < nu; ++it) {
+      sweep();
+      publish();
+    }
+    {
+      const Own8 r = own_apply<-1>(own_ld(B), c, v + at, s);
+      if (act) own_st(o + at, r);
+    }
+    __syncthreads();
+    {
+      float* bc = sm + L.vec[1];
+      each_node(5, tid, NT, [&](int i, int, int Xc, int Yc) {
+        const float* q = o + (2 * Yc + 2) * W + 4 + 2 * Xc + 1;   // fine node (2 Xc + 1, 2 Yc + 1)
+        float acc = 0.f;
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+          for (int dx = -1; dx <= 1; ++dx)
+            acc += ((dx == 0 ? 1.f : 0.5f) * (dy == 0 ? 1.f : 0.5f)) * q[dy * W + dx];
+        bc[i] = acc;
+      });
+    }
+    __syncthreads();
+    const float* xc = block_vcycle<float>(L, sm, nu, 1);   // ends with a block barrier
+    {
+      // coarse nodes 2 s' - 1 .. 2 s' + 1 beside each piece (s' = s, s + 8)
+      const int Yl = (min(y, NX - 1) + 1) >> 1;
+      const bool oy = y & 1;
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const float* q = xc + Yl * 33 + 2 * (s + 8 * g);
+        float c0 = q[0], c1 = q[1], c2 = q[2];
+        if (!oy) {
+          c0 = 0.5f * (c0 + q[33]);
+          c1 = 0.5f * (c1 + q[34]);
+          c2 = 0.5f * (c2 + q[35]);
+        }
+        cur.v[4 * g] += 0.5f * (c0 + c1);
+        cur.v[4 * g + 1] += c1;
+        cur.v[4 * g + 2] += 0.5f * (c1 + c2);
+        cur.v[4 * g + 3] += c2;
+      }
+      if (!act) cur = Own8{{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}};
+    }
+    publish();
+    for (int it = 0; it < nu; ++it) {
+      sweep();
+      if (it + 1 < nu) publish();
+    }
+    block_sum(red, own_dot(own_ld(B), cur), [&](double t) { scal_rho(S, t); });
+    {
+      const float beta = S.beta;
+      if (S.it > 0) {
+        const Own8 p = own_ld(P + at);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cur.v[i] = fmaf(beta, p.v[i], cur.v[i]);
+      }
+      if (act) own_st(P + at, cur);
+    }
+    __syncthreads();
+    Own8 q = own_apply<1>(Own8{{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}}, c, P + at, s);
+    block_sum(red, act ? own_dot(cur, q) : 0.f, [&](double t) { scal_alpha(S, t, a, true); });
+    if (S.done) break;
+    {
+      const float al = S.alpha;
+      Own8 u = own_ld(U), b = own_ld(B);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        u.v[i] = fmaf(al, cur.v[i], u.v[i]);
+        b.v[i] = fmaf(-al, q.v[i], b.v[i]);
+      }
+      own_st(U, u);
+      own_st(B, b);
+      block_sum(red, own_dot(b, b), [&](double t) { scal_conv(S, t, a, true); });
+    }
+  }
+  if (act) {
+    const Own8 u = own_ld(U);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int x = 4 * s + (i & 3) + (i >= 4 ? 32 : 0);
+      if (x < NX) dst[(size_t)(y * NX + x) * ldd + col] = (TD)u.v[i];
+    }
+  }
+  if (a.iters && tid == 0) a.iters[col] = S.it;
+}
+
 // ------------------------------------------------------------ host side ---
 
 // Blocks per column of k_block_diag: as many (up to MAX_C) as leave an SM to
@@ -606,12 +830,14 @@ static int diag_split(const sg_problem* h, const GridLevel& G, int w) {
   return C <= MAX_C && C <= G.ny ? C : 0;
 }
 
-static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L) {
+// Shared-memory layout of the grids from g0 on (0; 1 for k_block_vcycle63,
+// which keeps the finest one elsewhere, in `before` bytes).
+static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L, int g0 = 0, size_t before = 0) {
   L = BlockGrids{};
   L.G = (int)h->grids.size();
-  if (!h->mg_full || L.G > blk::MAX_GRIDS || h->grids[0].n > 1024) return false;
+  if (!h->mg_full || L.G <= g0 || L.G > blk::MAX_GRIDS || h->grids[g0].n > 1024) return false;
   int off = 0;
-  for (int g = 0; g < L.G; ++g) {
+  for (int g = g0; g < L.G; ++g) {
     const GridLevel& G = h->grids[g];
     int k = 0;
     while ((1 << k) < G.nx + 1) ++k;
@@ -625,9 +851,25 @@ static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L) {
     L.dinv[g] = es == 8 ? (const void*)G.dinv64 : (const void*)G.dinv32;
   }
   L.p = off;
-  off += (h->grids[0].nx + 2) * (h->grids[0].nx + 2);
+  if (g0 == 0) off += (h->grids[0].nx + 2) * (h->grids[0].nx + 2);
   L.total = off;
-  return (size_t)off * es <= (size_t)std::max(h->smem_optin, 48 * 1024) - 2048;
+  return before + (size_t)off * es <= (size_t)std::max(h->smem_optin, 48 * 1024) - 2048;
+}
+
+static bool layout63(const sg_problem* h, BlockGrids& L) {
+  return !h->grids.empty() && h->grids[0].planes &&
+         vcycle_layout(h, 4, L, 1, blk63::FLOATS * sizeof(float));
+}
+
+// FP32 V-cycle solves for which the block solvers are taken before the cluster
+// solver: every grid up to 63 x 63. sg_inner_solve with two steps, clusters and
+// blocks: 15 x 15 nodes 105 and 88 us (20 columns), 238 and 92 (715); 31 x 31
+// 121 and 100, 350 and 165; 63 x 63 134 and 112, 495 and 298. Faster at every
+// width from 1 to 1000, also where a wave of blocks is just begun.
+bool block_preferred(const sg_problem* h) {
+  if (h->block_off || h->grids.empty()) return false;
+  BlockGrids L;
+  return vcycle_layout(h, 4, L) || layout63(h, L);
 }
 
 bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o) {
@@ -639,7 +881,7 @@ bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o) 
     return C > 0 && ((size_t)(ceil_div(G.ny, C) + 2) * (G.nx + 2) + 6 * (size_t)G.nx) * es <= 40 * 1024;
   }
   BlockGrids L;
-  return vcycle_layout(h, dtype == SG_F64 ? 8 : 4, L);
+  return vcycle_layout(h, dtype == SG_F64 ? 8 : 4, L) || (dtype == SG_F32 && layout63(h, L));
 }
 
 template <typename TS, typename T, typename TD>
@@ -692,6 +934,16 @@ static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd
     return SG_OK;
   }
   BlockGrids L;
+  if constexpr (sizeof(T) == 4) {
+    if (layout63(h, L)) {
+      const size_t smem = (blk63::FLOATS + (size_t)L.total) * sizeof(float);
+      auto kern = k_block_vcycle63<TS, TD>;
+      SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      { kern<<<w, blk63::NT, smem, s>>>(a, L, (float)o.omega, o.nu, G.planes, src, lds, dst, ldd); note_launch(); }
+      SG_CHECK_LAUNCH();
+      return SG_OK;
+    }
+  }
   if (!vcycle_layout(h, sizeof(T), L)) {
     set_error("block inner solve: the hierarchy does not fit");
     return SG_ERR_UNSUPPORTED;

@@ -1307,6 +1307,7 @@ static int cluster_path(const sg_problem* h, int dtype, int w) {
   if (dtype != SG_F32 || !cs) return 0;
   const auto it = h->inner_pick.find(w);
   if (it != h->inner_pick.end() && path_eligible(cs, w, it->second)) return it->second;
+  if (block_preferred(h)) return 0;
   for (int path : {3, 1, 2})
     if (path_eligible(cs, w, path)) return path;
   return 0;

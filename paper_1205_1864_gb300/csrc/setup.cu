@@ -60,13 +60,24 @@ static int upload(T** dst, const T* src, size_t count) {
   return SG_OK;
 }
 
-// FP32 stencils [n][9] and inverse diagonals into 48-byte records (GridLevel::st12)
-__global__ void k_pack_stencil(int n, const float* __restrict__ st, const float* __restrict__ dinv,
-                               float* __restrict__ st12) {
+// FP32 stencils [n][9] and inverse diagonals into 48-byte records and planes
+// (GridLevel::st12, planes)
+__global__ void k_pack_stencil(int nx, int ny, const float* __restrict__ st, const float* __restrict__ dinv,
+                               float* __restrict__ st12, float* __restrict__ planes) {
+  const int n = nx * ny;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * 12; i += gridDim.x * blockDim.x) {
     const int node = i / 12, e = i - node * 12, c = e & 3;
-    st12[i] = c < 3 ? st[node * 9 + e / 4 * 3 + c] : (e == 11 ? dinv[node] : 0.f);
+    const float v = c < 3 ? st[node * 9 + e / 4 * 3 + c] : (e == 11 ? dinv[node] : 0.f);
+    st12[i] = v;
+    const int plane = c < 3 ? e / 4 * 3 + c : (e == 11 ? 9 : -1);
+    if (planes && plane >= 0) planes[(plane * ny + node / nx) * (nx + 1) + node % nx] = v;
   }
+}
+
+int pack_stencils(GridLevel& g) {
+  { k_pack_stencil<<<std::min((g.n * 12 + 255) / 256, 4096), 256>>>(g.nx, g.ny, g.st32, g.dinv32, g.st12, g.planes); ::sghsc::note_launch(); }
+  SG_CHECK_LAUNCH();
+  return SG_OK;
 }
 
 struct HostEdges {
@@ -384,7 +395,7 @@ static void galerkin_coarsen(int nx, int ny, const std::vector<double>& st, int 
   }
 }
 
-static int upload_grid(GridLevel& g, const std::vector<double>& st) {
+static int upload_grid(GridLevel& g, const std::vector<double>& st, bool finest) {
   SG_TRY(upload(&g.st_base, st.data(), st.size()));
   std::vector<float> st32(st.begin(), st.end());
   std::vector<double> dinv(g.n);
@@ -395,8 +406,11 @@ static int upload_grid(GridLevel& g, const std::vector<double>& st) {
   SG_TRY(upload(&g.dinv64, dinv.data(), dinv.size()));
   SG_TRY(upload(&g.dinv32, dinv32.data(), dinv32.size()));
   SG_TRY_CUDA(cudaMalloc((void**)&g.st12, dinv32.size() * 12 * sizeof(float)));
-  { k_pack_stencil<<<std::min(((int)dinv32.size() * 12 + 255) / 256, 4096), 256>>>((int)dinv32.size(), g.st32, g.dinv32, g.st12); ::sghsc::note_launch(); }
-  SG_CHECK_LAUNCH();
+  if (finest && g.nx == 63 && g.ny == 63) {
+    SG_TRY_CUDA(cudaMalloc((void**)&g.planes, 10 * 63 * 64 * sizeof(float)));
+    SG_TRY_CUDA(cudaMemset(g.planes, 0, 10 * 63 * 64 * sizeof(float)));
+  }
+  SG_TRY(pack_stencils(g));
   return SG_OK;
 }
 
@@ -563,7 +577,7 @@ static int setup_impl(const sg_mesh* mesh, int M, int p, int family, int n, int 
       while (true) {
         GridLevel g;
         g.nx = gx; g.ny = gy; g.n = gx * gy;
-        SG_TRY(upload_grid(g, st));
+        SG_TRY(upload_grid(g, st, h->grids.empty()));
         h->grids.push_back(g);
         if (!pow2) break;            // the finest grid alone: diagonal M_0 only
         if (gx <= 1) {
@@ -625,17 +639,14 @@ __global__ void k_scale_vals(long long count, int M1, const double* __restrict__
 
 // multigrid stencils of s * A_0: st = s * base, dinv = 1 / (s * base_centre)
 __global__ void k_scale_grid(int n, const double* __restrict__ base, double s, double* __restrict__ st64,
-                             float* __restrict__ st32, double* __restrict__ dinv64, float* __restrict__ dinv32,
-                             float* __restrict__ st12) {
+                             float* __restrict__ st32, double* __restrict__ dinv64, float* __restrict__ dinv32) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * 9; i += gridDim.x * blockDim.x) {
     const double v = s * base[i];
     st64[i] = v;
     st32[i] = (float)v;
-    st12[i / 9 * 12 + i % 9 / 3 * 4 + i % 3] = (float)v;
     if (i % 9 == 4) {
       dinv64[i / 9] = 1.0 / v;
       dinv32[i / 9] = (float)(1.0 / v);
-      st12[i / 9 * 12 + 11] = (float)(1.0 / v);
     }
   }
 }
@@ -667,7 +678,8 @@ int sg_set_scales(sg_problem* h, const double* scale) {
   const long long count = (long long)h->nnz * h->nterm;
   { k_scale_vals<<<(int)std::min<long long>((count + 255) / 256, 4096), 256>>>(count, h->nterm, h->vals_base, h->scales_dev, h->vals64, h->vals32, (df64*)h->vals_df); ::sghsc::note_launch(); }
   for (auto& g : h->grids)
-    { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g.n, g.st_base, scale[0], g.st64, g.st32, g.dinv64, g.dinv32, g.st12); ::sghsc::note_launch(); }
+    { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g.n, g.st_base, scale[0], g.st64, g.st32, g.dinv64, g.dinv32); ::sghsc::note_launch(); }
+  for (auto& g : h->grids) SG_TRY(pack_stencils(g));
   SG_TRY_CUDA(cudaGetLastError());
   SG_TRY_CUDA(cudaDeviceSynchronize());
   return SG_OK;
@@ -765,7 +777,7 @@ void sg_destroy(sg_problem* h) {
   free_edges(h->sub);
   for (auto& e : h->dlev) free_edges(e);
   for (auto& g : h->grids) {
-    cudaFree(g.st_base); cudaFree(g.st64); cudaFree(g.st32); cudaFree(g.dinv64); cudaFree(g.dinv32); cudaFree(g.st12);
+    cudaFree(g.st_base); cudaFree(g.st64); cudaFree(g.st32); cudaFree(g.dinv64); cudaFree(g.dinv32); cudaFree(g.st12); cudaFree(g.planes);
   }
   if (h->cap[0]) cudaDeviceSynchronize();
   clear_graphs(h);

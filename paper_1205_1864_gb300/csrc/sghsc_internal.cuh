@@ -107,6 +107,9 @@ struct GridLevel {
   // FP32 stencil and inverse diagonal of a node in 48 bytes, three 16-byte
   // pieces: the row above, the own row, the row below with dinv in its last slot
   float* st12 = nullptr;
+  // on a finest grid of 63 x 63: the nine coefficients and the inverse diagonal
+  // as planes [10][63][64] (rows of 64: whole 16-byte pieces), else null
+  float* planes = nullptr;
 };
 
 // Device control block of one batched inner solve.
@@ -292,6 +295,9 @@ bool rows32_usable(const sg_problem* h, const EdgeList& E, int wx, bool diag);
 int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, int ldx, int wx, const float* Yin,
                   int ldyin, float* Y, int ldy, cudaStream_t s);
 
+// The FP32 stencil copies of a grid (st12, planes) from st32 and dinv32.
+int pack_stencils(GridLevel& g);
+
 // ---- inner solver (inner.cu) ----
 int ensure_inner_work(sg_problem* h, int dtype, int wcap);
 void free_inner_work(sg_problem* h);
@@ -325,9 +331,11 @@ int inner_solve_cluster(sg_problem* h, const void* src, int ld_src, int src_t, v
                         int w, const sg_prec_opts& o, cudaStream_t s);
 
 // ---- inner solver on small grids, one launch per solve (inner_block.cu) ----
-// Batches the cluster solver does not take: any grid that a cluster of
-// blocks holds with the diagonal M_0, at most 1024 nodes with the V-cycle.
+// Any grid that a cluster of blocks holds with the diagonal M_0; with the
+// V-cycle at most 1024 nodes, and 63 x 63 in FP32.
 bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o);
+// True when FP32 V-cycle solves on h take it before the cluster solver.
+bool block_preferred(const sg_problem* h);
 int inner_solve_block(sg_problem* h, int dtype, const void* src, int ld_src, int src_t, void* dst, int ld_dst,
                       int dst_t, int w, const sg_prec_opts& o, cudaStream_t s);
 

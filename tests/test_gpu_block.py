@@ -8,7 +8,8 @@ order of sums. After k steps the iterates differ by about k u times the
 condition of the preconditioned matrix (below 2 with the V-cycle, below the
 number of nodes with the diagonal), relative to the largest entry: 1e-11 in
 FP64 (u = 1.1e-16, 4 steps, up to 8281 nodes: 4e-12), 2e-3 in FP32 with the
-diagonal and 2e-5 with the V-cycle."""
+diagonal and 2e-5 with the V-cycle (1e-4 on 63 x 63 nodes, the bar of the other
+solvers there: A_0 itself is rounded, which its small eigenvalues feel)."""
 import numpy as np
 import pytest
 
@@ -37,7 +38,7 @@ def _handles(lib, monkeypatch, ne):
 @pytest.mark.parametrize("m0,ne,w", [("diag", 2, 1), ("diag", 5, 3), ("diag", 10, 40), ("diag", 17, 7), ("diag", 30, 1),
                                      ("diag", 30, 35), ("diag", 33, 160), ("diag", 64, 2), ("diag", 91, 5),
                                      ("diag", 92, 3), ("vcycle", 2, 2), ("vcycle", 4, 3), ("vcycle", 8, 1),
-                                     ("vcycle", 16, 20), ("vcycle", 32, 155)])
+                                     ("vcycle", 16, 20), ("vcycle", 32, 155), ("vcycle", 64, 3), ("vcycle", 64, 160)])
 def test_block_solver_matches_oracle(lib, monkeypatch, m0, ne, w, prec):
     import torch
     dt, code = (torch.float64, lib.SG_F64) if prec == "fp64" else (torch.float32, lib.SG_F32)
@@ -62,7 +63,7 @@ def test_block_solver_matches_oracle(lib, monkeypatch, m0, ne, w, prec):
     o = lib.prec_opts(precision=code, m0=kind, inner_fixed_iters=steps)
     X, it = lib.sg_inner_solve(h, Bt, o)
     ref = krylov.pcg_columns(lambda v: A[0] @ v, B.astype(np.float64), pre, tol=0.0, maxit=steps, fixed_iters=steps)[0]
-    tol = 1e-11 if prec == "fp64" else (2e-3 if m0 == "diag" else 2e-5)
+    tol = 1e-11 if prec == "fp64" else (2e-3 if m0 == "diag" else 1e-4 if ne == 64 else 2e-5)
     assert np.abs(X.double().cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
     assert all(it[c] == (0 if w > 2 and c == 1 else steps) for c in range(w))
     # to a tolerance: the same counts as the stand-alone kernels
