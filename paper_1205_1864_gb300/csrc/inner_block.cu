@@ -35,7 +35,7 @@
 // V-cycle 15 x 15, FP64, 20 columns 251 -> 104, 31 x 31, FP32, 300 columns
 // 229 -> 120. No size it can hold was slower (1 to 1000 columns, both
 // types), so every batch that fits takes it. Whole FP64 solves: 16 x 16
-// elements, M = 3, p = 3, 6.64 -> 1.75 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
+// elements, M = 3, p = 3, 6.64 -> 1.40 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
 // 274 -> 15.4 ms; lognormal 10 x 10, M = 3, p = 3, 1034 -> 77.6 ms.
 #include <cooperative_groups.h>
 
@@ -353,14 +353,33 @@ __global__ void __launch_bounds__(blk::NT) k_block_diag(BlockArgs a, const T* __
 // The hierarchy in shared memory: per grid (nx = ny = 2^k - 1, row stride
 // W = nx + 2) the vectors b, x, y with zero borders, the stencils [n][9] and
 // the inverse diagonal [n]; on the finest grid also p (with borders).
+//
+// With the default smoothing everything from the 7 x 7 grid down is one dense
+// matrix on that grid's right-hand side (grid gm; -1: none): 13 phases of one
+// to two warps, each a chain of a stencil's multiply-adds, are one phase of
+// 49 / LP of them: 16 x 16 elements, M = 3, p = 3, FP64, whole solve 1.75 ->
+// 1.40 ms; a step on 63 x 63 nodes, FP32, 17 -> 12.5 us.
 struct BlockGrids {
-  int G;
+  int G, gm;
   int k[blk::MAX_GRIDS];                       // nx + 1 = 2^k
   int vec[blk::MAX_GRIDS], coef[blk::MAX_GRIDS];   // element offsets of b (x, y follow) and of the stencils
   int p, total;                                // offset of p, elements in all
-  const void* st[blk::MAX_GRIDS];
+  const void* st[blk::MAX_GRIDS];   // (of grid gm: its matrix)
   const void* dinv[blk::MAX_GRIDS];
 };
+
+// The matrix of grid gm: LP threads per row, each every LP-th column; rows are
+// padded with zeros to whole turns (odd multiples of LP in banks: no two lanes
+// of a warp in one bank). The right-hand side lies compact before the padded
+// solution.
+namespace cmx {
+constexpr int N = 49, W = 9;
+__host__ __device__ constexpr int lp(int threads) { return threads / 64; }
+__host__ __device__ constexpr int stride(int lp) { return (N + lp - 1) / lp * lp; }
+constexpr int B = 56;                     // the longest row
+constexpr int VECS = B + W * W;
+constexpr int COEFS = N * B;
+}  // namespace cmx
 
 // f(padded index, node) over the nodes of a grid of nx + 1 = 2^k, by the
 // threads t, t + nt, ... (columns of 2^k: the last of each row is skipped)
@@ -393,11 +412,52 @@ __device__ __forceinline__ void phase_sync(bool wm) {
   else __syncthreads();
 }
 
+// Zero vectors and the coefficients of the grids from g0 on (not yet visible
+// to the other threads of the block); om: the damping.
+template <typename T>
+__device__ __forceinline__ void stage_grids(const BlockGrids& L, T* sm, T om, int g0 = 0) {
+  const int tid = threadIdx.x, NT = blockDim.x;
+  for (int g = g0; g < L.G; ++g) {
+    const T* gs = (const T*)L.st[g];
+    if (g == L.gm) {
+      const int S = cmx::stride(cmx::lp(NT));
+      for (int i = tid; i < cmx::VECS; i += NT) sm[L.vec[g] + i] = T(0);
+      for (int i = tid; i < cmx::N * S; i += NT) {
+        const int r = i / S, c = i - r * S;
+        sm[L.coef[g] + i] = c < cmx::N ? gs[r * cmx::N + c] : T(0);
+      }
+      return;
+    }
+    const int Wg = (1 << L.k[g]) + 1, ng = (Wg - 2) * (Wg - 2);
+    for (int i = tid; i < 3 * Wg * Wg; i += NT) sm[L.vec[g] + i] = T(0);
+    const T* gd = (const T*)L.dinv[g];
+    for (int i = tid; i < 9 * ng; i += NT) sm[L.coef[g] + i] = gs[i];
+    // the damped inverse diagonal (the plain one on the one-node grid, solved exactly)
+    for (int i = tid; i < ng; i += NT) sm[L.coef[g] + 9 * ng + i] = g == L.G - 1 ? gd[i] : om * gd[i];
+  }
+}
+
+// x = M b on grid gm
+template <typename T, int LP>
+__device__ __forceinline__ void apply_cmat(const T* M, const T* b, T* x) {
+  constexpr int S = cmx::stride(LP);
+  const int r = threadIdx.x / LP, l = threadIdx.x % LP;
+  if (threadIdx.x / 32 > (cmx::N - 1) * LP / 32) return;   // whole warps
+  const T* m = M + min(r, cmx::N - 1) * S + l;
+  T acc = T(0);
+#pragma unroll
+  for (int j = 0; j < S / LP; ++j) acc = fma(m[j * LP], b[j * LP + l], acc);
+#pragma unroll
+  for (int o = LP / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (l == 0 && r < cmx::N) x[(r / 7 + 1) * cmx::W + r % 7 + 1] = acc;
+}
+
 // One V-cycle from grid g0's b; returns the buffer that holds the result.
 // Every thread of the block calls it.
 template <typename T>
 __device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu, int g0 = 0) {
-  const int tid = threadIdx.x, G = L.G;
+  const int tid = threadIdx.x;
+  const int G = L.gm < 0 ? L.G : L.gm + 1;
   auto wmode = [&](int g) { return L.k[g] <= 2 && g > 0; };
   auto vsize = [&](int g) { const int W = (1 << L.k[g]) + 1; return W * W; };
   auto odd = [&](int s) { return (s & 1) != 0; };
@@ -411,6 +471,14 @@ __device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu, int g0 = 0) {
     const T* b = sm + L.vec[g];
     T* c = sm + L.vec[g] + V;
     T* o = c + V;
+    if (g == L.gm) {
+      T* x = sm + L.vec[g] + cmx::B;
+      if (blockDim.x == 128) apply_cmat<T, 2>(st, b, x);
+      else if (blockDim.x == 256) apply_cmat<T, 4>(st, b, x);
+      else apply_cmat<T, 8>(st, b, x);
+      __syncthreads();
+      break;
+    }
     if (!wm || tid < 32) {
       if (g == G - 1) {   // one node: exact
         each_node(k, tid, nt, [&](int i, int node, int, int) { c[i] = di[node] * b[i]; });
@@ -428,7 +496,8 @@ __device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu, int g0 = 0) {
         each_node(k, tid, nt, [&](int i, int node, int, int) { o[i] = dot9<-1>(b[i], st + 9 * node, c, i, W); });
         phase_sync(wm);
         T* bc = sm + L.vec[g + 1];
-        each_node(L.k[g + 1], tid, nt, [&](int i, int, int X, int Y) {
+        const bool compact = g + 1 == L.gm;
+        each_node(L.k[g + 1], tid, nt, [&](int i, int node, int X, int Y) {
           const T* f = o + (2 * Y + 2) * W + 2 * X + 2;   // fine node (2X + 1, 2Y + 1)
           T acc = T(0);
 #pragma unroll
@@ -436,13 +505,13 @@ __device__ T* block_vcycle(const BlockGrids& L, T* sm, int nu, int g0 = 0) {
 #pragma unroll
             for (int dx = -1; dx <= 1; ++dx)
               acc += ((dx == 0 ? T(1) : T(0.5)) * (dy == 0 ? T(1) : T(0.5))) * f[dy * W + dx];
-          bc[i] = acc;
+          bc[compact ? node : i] = acc;
         });
         phase_sync(wm);
       }
     }
   }
-  T* res = sm + L.vec[G - 1] + vsize(G - 1);
+  T* res = sm + L.vec[G - 1] + (L.gm < 0 ? vsize(G - 1) : cmx::B);
   for (int g = G - 2; g >= g0; --g) {
     const int W = (1 << L.k[g]) + 1, V = vsize(g), k = L.k[g], n = (W - 2) * (W - 2);
     const int Wc = (1 << L.k[g + 1]) + 1;
@@ -526,15 +595,7 @@ __global__ void __launch_bounds__(blk::VNT) k_block_vcycle(BlockArgs a, BlockGri
     pc[u] = in ? (y + 1) * W + xx + 1 : W + 1;
     x[u] = p[u] = q[u] = T(0);
   }
-  for (int g = 0; g < L.G; ++g) {
-    const int Wg = (1 << L.k[g]) + 1, ng = (Wg - 2) * (Wg - 2);
-    for (int i = tid; i < 3 * Wg * Wg; i += NT) sm[L.vec[g] + i] = T(0);
-    const T* gs = (const T*)L.st[g];
-    const T* gd = (const T*)L.dinv[g];
-    for (int i = tid; i < 9 * ng; i += NT) sm[L.coef[g] + i] = gs[i];
-    // the damped inverse diagonal (the plain one on the one-node grid, solved exactly)
-    for (int i = tid; i < ng; i += NT) sm[L.coef[g] + 9 * ng + i] = g == L.G - 1 ? gd[i] : om * gd[i];
-  }
+  stage_grids<T>(L, sm, om);
   for (int i = tid; i < V; i += NT) ps[i] = T(0);
   __syncthreads();
   {
@@ -600,8 +661,7 @@ __global__ void __launch_bounds__(blk::VNT) k_block_vcycle(BlockArgs a, BlockGri
 // and 32 + 4 s .. of row y: a row is read as two 16-byte pieces per thread, the
 // neighbours beside them come from the lanes beside it. The coarse grids run
 // in shared memory through block_vcycle. What bounds it: the barriers and the
-// chains between them (a step is 17 us, some 8 of them on the 31 x 31 grid and
-// below). Read node by node, the stencils took 4 us of a solve of two steps;
+// chains between them (a step is 12.5 us, half of it on the coarse grids). Read node by node, the stencils took 4 us of a solve of two steps;
 // from planes with rows of 64 they are whole lines.
 namespace blk63 {
 constexpr int NT = 512, NX = 63;
@@ -675,14 +735,7 @@ __global__ void __launch_bounds__(blk63::NT, 1)
   float* const D = B + OWN;
   float* const U = D + OWN;
   for (int i = tid; i < 3 * VEC; i += NT) X[i] = 0.f;
-  for (int g = 1; g < L.G; ++g) {
-    const int Wg = (1 << L.k[g]) + 1, ng = (Wg - 2) * (Wg - 2);
-    for (int i = tid; i < 3 * Wg * Wg; i += NT) sm[L.vec[g] + i] = 0.f;
-    const float* gs = (const float*)L.st[g];
-    const float* gd = (const float*)L.dinv[g];
-    for (int i = tid; i < 9 * ng; i += NT) sm[L.coef[g] + i] = gs[i];
-    for (int i = tid; i < ng; i += NT) sm[L.coef[g] + 9 * ng + i] = g == L.G - 1 ? gd[i] : om * gd[i];
-  }
+  stage_grids<float>(L, sm, om, 1);
   float c[8][9];
   {
     Own8 b;
@@ -832,9 +885,12 @@ static int diag_split(const sg_problem* h, const GridLevel& G, int w) {
 
 // Shared-memory layout of the grids from g0 on (0; 1 for k_block_vcycle63,
 // which keeps the finest one elsewhere, in `before` bytes).
-static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L, int g0 = 0, size_t before = 0) {
+static bool vcycle_layout(const sg_problem* h, size_t es, const sg_prec_opts& o, BlockGrids& L, int g0 = 0,
+                          size_t before = 0) {
   L = BlockGrids{};
   L.G = (int)h->grids.size();
+  L.gm = h->cmat_base && o.nu == 2 && o.omega == 0.8 ? L.G - 3 : -1;   // (7 x 7, 3 x 3 and one node)
+
   if (!h->mg_full || L.G <= g0 || L.G > blk::MAX_GRIDS || h->grids[g0].n > 1024) return false;
   int off = 0;
   for (int g = g0; g < L.G; ++g) {
@@ -844,6 +900,13 @@ static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L, int g0 
     if (G.nx != G.ny || (1 << k) != G.nx + 1) return false;
     L.k[g] = k;
     L.vec[g] = off;
+    if (g == L.gm) {
+      off += cmx::VECS;
+      L.coef[g] = off;
+      off += cmx::COEFS;
+      L.st[g] = es == 8 ? (const void*)h->cmat64 : (const void*)h->cmat32;
+      break;
+    }
     off += 3 * (G.nx + 2) * (G.nx + 2);
     L.coef[g] = off;
     off += 10 * G.n;
@@ -856,9 +919,9 @@ static bool vcycle_layout(const sg_problem* h, size_t es, BlockGrids& L, int g0 
   return before + (size_t)off * es <= (size_t)std::max(h->smem_optin, 48 * 1024) - 2048;
 }
 
-static bool layout63(const sg_problem* h, BlockGrids& L) {
+static bool layout63(const sg_problem* h, const sg_prec_opts& o, BlockGrids& L) {
   return !h->grids.empty() && h->grids[0].planes &&
-         vcycle_layout(h, 4, L, 1, blk63::FLOATS * sizeof(float));
+         vcycle_layout(h, 4, o, L, 1, blk63::FLOATS * sizeof(float));
 }
 
 // FP32 V-cycle solves for which the block solvers are taken before the cluster
@@ -868,8 +931,10 @@ static bool layout63(const sg_problem* h, BlockGrids& L) {
 // width from 1 to 1000, also where a wave of blocks is just begun.
 bool block_preferred(const sg_problem* h) {
   if (h->block_off || h->grids.empty()) return false;
+  sg_prec_opts o;   // the default smoothing: the larger layout
+  sg_default_prec_opts(&o);
   BlockGrids L;
-  return vcycle_layout(h, 4, L) || layout63(h, L);
+  return vcycle_layout(h, 4, o, L) || layout63(h, o, L);
 }
 
 bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o) {
@@ -881,7 +946,7 @@ bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o) 
     return C > 0 && ((size_t)(ceil_div(G.ny, C) + 2) * (G.nx + 2) + 6 * (size_t)G.nx) * es <= 40 * 1024;
   }
   BlockGrids L;
-  return vcycle_layout(h, dtype == SG_F64 ? 8 : 4, L) || (dtype == SG_F32 && layout63(h, L));
+  return vcycle_layout(h, dtype == SG_F64 ? 8 : 4, o, L) || (dtype == SG_F32 && layout63(h, o, L));
 }
 
 template <typename TS, typename T, typename TD>
@@ -935,7 +1000,7 @@ static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd
   }
   BlockGrids L;
   if constexpr (sizeof(T) == 4) {
-    if (layout63(h, L)) {
+    if (layout63(h, o, L)) {
       const size_t smem = (blk63::FLOATS + (size_t)L.total) * sizeof(float);
       auto kern = k_block_vcycle63<TS, TD>;
       SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -944,7 +1009,7 @@ static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd
       return SG_OK;
     }
   }
-  if (!vcycle_layout(h, sizeof(T), L)) {
+  if (!vcycle_layout(h, sizeof(T), o, L)) {
     set_error("block inner solve: the hierarchy does not fit");
     return SG_ERR_UNSUPPORTED;
   }

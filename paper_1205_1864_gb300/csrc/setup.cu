@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <algorithm>
+#include <functional>
 #include <atomic>
 #include <map>
 
@@ -395,6 +396,57 @@ static void galerkin_coarsen(int nx, int ny, const std::vector<double>& st, int 
   }
 }
 
+// The matrix of one V-cycle (two damped Jacobi sweeps, omega 0.8, before and
+// after; the one-node grid exactly) on a grid of nx x nx nodes; st: the
+// stencils of this grid and of all below it. Column by column, in FP64.
+static std::vector<double> vcycle_matrix(int nx, const std::vector<std::vector<double>>& st) {
+  const int n = nx * nx;
+  std::vector<double> M((size_t)n * n);
+  std::function<std::vector<double>(size_t, int, const std::vector<double>&)> cycle =
+      [&](size_t g, int m, const std::vector<double>& b) {
+        const auto& s9 = st[g];
+        auto at = [&](const std::vector<double>& v, int x, int y, int w) {
+          return x < 0 || y < 0 || x >= w || y >= w ? 0.0 : v[y * w + x];
+        };
+        auto residual = [&](const std::vector<double>& x) {
+          std::vector<double> r(b);
+          for (int i = 0; i < m * m; ++i)
+            for (int e = 0; e < 9; ++e) r[i] -= s9[i * 9 + e] * at(x, i % m + e % 3 - 1, i / m + e / 3 - 1, m);
+          return r;
+        };
+        std::vector<double> x(m * m, 0.0);
+        if (m == 1) {
+          x[0] = b[0] / s9[4];
+          return x;
+        }
+        auto sweep = [&]() {
+          const auto r = residual(x);
+          for (int i = 0; i < m * m; ++i) x[i] += 0.8 / s9[i * 9 + 4] * r[i];
+        };
+        for (int k = 0; k < 2; ++k) sweep();
+        const auto r = residual(x);
+        const int mc = (m - 1) / 2;
+        std::vector<double> bc(mc * mc, 0.0);
+        auto weight = [](int d) { return d == 0 ? 1.0 : 0.5; };
+        for (int c = 0; c < mc * mc; ++c)
+          for (int e = 0; e < 9; ++e)
+            bc[c] += weight(e % 3 - 1) * weight(e / 3 - 1) * at(r, 2 * (c % mc) + e % 3, 2 * (c / mc) + e / 3, m);
+        const auto xc = cycle(g + 1, mc, bc);
+        for (int c = 0; c < mc * mc; ++c)
+          for (int e = 0; e < 9; ++e)
+            x[(2 * (c / mc) + e / 3) * m + 2 * (c % mc) + e % 3] += weight(e % 3 - 1) * weight(e / 3 - 1) * xc[c];
+        for (int k = 0; k < 2; ++k) sweep();
+        return x;
+      };
+  for (int j = 0; j < n; ++j) {
+    std::vector<double> b(n, 0.0);
+    b[j] = 1.0;
+    const auto x = cycle(0, nx, b);
+    for (int i = 0; i < n; ++i) M[(size_t)i * n + j] = x[i];
+  }
+  return M;
+}
+
 static int upload_grid(GridLevel& g, const std::vector<double>& st, bool finest) {
   SG_TRY(upload(&g.st_base, st.data(), st.size()));
   std::vector<float> st32(st.begin(), st.end());
@@ -574,7 +626,9 @@ static int setup_impl(const sg_mesh* mesh, int M, int p, int family, int n, int 
       h->nx = nx;
       h->ny = ny;
       int gx = nx, gy = ny;
+      std::vector<std::vector<double>> small;   // stencils from the 7 x 7 grid on
       while (true) {
+        if (pow2 && gx <= 7 && nx > 7) small.push_back(st);
         GridLevel g;
         g.nx = gx; g.ny = gy; g.n = gx * gy;
         SG_TRY(upload_grid(g, st, h->grids.empty()));
@@ -582,6 +636,13 @@ static int setup_impl(const sg_mesh* mesh, int M, int p, int family, int n, int 
         if (!pow2) break;            // the finest grid alone: diagonal M_0 only
         if (gx <= 1) {
           h->mg_full = true;
+          if (!small.empty()) {
+            const std::vector<double> M = vcycle_matrix(7, small);
+            const std::vector<float> M32(M.begin(), M.end());
+            SG_TRY(upload(&h->cmat_base, M.data(), M.size()));
+            SG_TRY(upload(&h->cmat64, M.data(), M.size()));
+            SG_TRY(upload(&h->cmat32, M32.data(), M32.size()));
+          }
           break;
         }
         const int nxc = (gx - 1) / 2, nyc = (gy - 1) / 2;
@@ -637,6 +698,16 @@ __global__ void k_scale_vals(long long count, int M1, const double* __restrict__
   }
 }
 
+// the V-cycle matrix of s * A_0: that of A_0 divided by s
+__global__ void k_scale_cmat(int n, const double* __restrict__ base, double s, double* __restrict__ m64,
+                             float* __restrict__ m32) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double v = base[i] / s;
+    m64[i] = v;
+    m32[i] = (float)v;
+  }
+}
+
 // multigrid stencils of s * A_0: st = s * base, dinv = 1 / (s * base_centre)
 __global__ void k_scale_grid(int n, const double* __restrict__ base, double s, double* __restrict__ st64,
                              float* __restrict__ st32, double* __restrict__ dinv64, float* __restrict__ dinv32) {
@@ -680,6 +751,8 @@ int sg_set_scales(sg_problem* h, const double* scale) {
   for (auto& g : h->grids)
     { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g.n, g.st_base, scale[0], g.st64, g.st32, g.dinv64, g.dinv32); ::sghsc::note_launch(); }
   for (auto& g : h->grids) SG_TRY(pack_stencils(g));
+  if (h->cmat_base)
+    { k_scale_cmat<<<10, 256>>>(49 * 49, h->cmat_base, scale[0], h->cmat64, h->cmat32); ::sghsc::note_launch(); }
   SG_TRY_CUDA(cudaGetLastError());
   SG_TRY_CUDA(cudaDeviceSynchronize());
   return SG_OK;
@@ -776,6 +849,7 @@ void sg_destroy(sg_problem* h) {
   for (auto& e : h->post) free_edges(e);
   free_edges(h->sub);
   for (auto& e : h->dlev) free_edges(e);
+  cudaFree(h->cmat_base); cudaFree(h->cmat64); cudaFree(h->cmat32);
   for (auto& g : h->grids) {
     cudaFree(g.st_base); cudaFree(g.st64); cudaFree(g.st32); cudaFree(g.dinv64); cudaFree(g.dinv32); cudaFree(g.st12); cudaFree(g.planes);
   }

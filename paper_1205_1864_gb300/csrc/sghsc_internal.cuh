@@ -189,6 +189,12 @@ struct sg_problem {
   double* fG = nullptr;                     // n x off[p] right-hand side g_{p-1} of the reduced system
   // multigrid
   std::vector<sghsc::GridLevel> grids;
+  // One V-cycle of the default smoothing (nu 2, omega 0.8) from the 7 x 7 grid
+  // down as a matrix [49][49] on that grid's right-hand side: of A_0 at scale 1,
+  // and at the present scale; null when the finest grid is no larger.
+  double* cmat_base = nullptr;
+  double* cmat64 = nullptr;
+  float* cmat32 = nullptr;
   bool mg_full = false;                     // the hierarchy reaches the one-node grid (V-cycle usable)
   int cb_level = 0;                         // first grid handled by the in-block coarse V-cycle
   void* cl_plan = nullptr;                  // cluster inner solvers: plans and scratch (null: not usable)

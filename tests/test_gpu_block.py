@@ -75,3 +75,25 @@ def test_block_solver_matches_oracle(lib, monkeypatch, m0, ne, w, prec):
         assert float((X - X0).abs().max()) <= 1e-9 * float(X0.abs().max())
     else:   # a residual at the threshold may stop one step apart
         assert int(np.abs(it - it0).max()) <= 1
+
+
+@pytest.mark.parametrize("ne,prec,tol", [(16, "fp64", 1e-13), (32, "fp64", 1e-13), (16, "fp32", 1e-5), (32, "fp32", 1e-5),
+                                         (64, "fp32", 1e-5)])
+def test_coarse_matrix_equals_the_smoothed_cycle(lib, monkeypatch, ne, prec, tol):
+    """The matrix of the grids from 7 x 7 down (the default smoothing) against
+    the grid-by-grid cycle, which a damping one rounding away still takes, also
+    after a change of scale. One step: the two differ by the rounding of some 60
+    operations a node, 1e-14 in FP64 and 4e-6 in FP32."""
+    import torch
+    prob, A, h, _ = _handles(lib, monkeypatch, ne)
+    dt, code = (torch.float64, lib.SG_F64) if prec == "fp64" else (torch.float32, lib.SG_F32)
+    B = torch.tensor(S.random_block(prob.n, 5, seed=ne), dtype=dt, device="cuda")
+    for scale in (1.0, 3.0):
+        lib.sg_set_scales(h, np.full(2, scale))
+        X = [lib.sg_inner_solve(h, B, lib.prec_opts(precision=code, inner_fixed_iters=1, omega=om))[0]
+             for om in (0.8, float(np.nextafter(0.8, 1)))]
+        assert float((X[0] - X[1]).abs().max()) <= tol * float(X[1].abs().max())
+        ref = krylov.pcg_columns(lambda v: scale * (A[0] @ v), B.double().cpu().numpy(),
+                                 lambda r: gmg.vcycle(gmg.hierarchy(scale * A[0], ne), r), tol=0.0, maxit=1,
+                                 fixed_iters=1)[0]
+        assert np.abs(X[0].double().cpu().numpy() - ref).max() <= (1e-12 if prec == "fp64" else 1e-4) * np.abs(ref).max()
