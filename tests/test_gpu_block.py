@@ -97,3 +97,16 @@ def test_coarse_matrix_equals_the_smoothed_cycle(lib, monkeypatch, ne, prec, tol
                                  lambda r: gmg.vcycle(gmg.hierarchy(scale * A[0], ne), r), tol=0.0, maxit=1,
                                  fixed_iters=1)[0]
         assert np.abs(X[0].double().cpu().numpy() - ref).max() <= (1e-12 if prec == "fp64" else 1e-4) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("w", [5, 40, 100])
+def test_coarse_matrix_on_clusters(lib, w):
+    """The same in the cluster solvers (127 x 127 nodes; clusters of 16 and 8
+    blocks, finest grid in global memory): one step, 1e-5."""
+    import torch
+    prob, A, _, _ = problem(128, 1, 1)
+    h = lib.SGProblem.from_inputs(prob, 1)
+    B = torch.tensor(S.random_block(prob.n, w, seed=w), dtype=torch.float32, device="cuda")
+    X = [lib.sg_inner_solve(h, B, lib.prec_opts(precision=lib.SG_F32, inner_fixed_iters=1, omega=om))[0]
+         for om in (0.8, float(np.nextafter(0.8, 1)))]
+    assert float((X[0] - X[1]).abs().max()) <= 1e-5 * float(X[1].abs().max())
