@@ -7,7 +7,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <algorithm>
-#include <functional>
 #include <atomic>
 #include <map>
 
@@ -397,54 +396,55 @@ static void galerkin_coarsen(int nx, int ny, const std::vector<double>& st, int 
 }
 
 // The matrix of one V-cycle (two damped Jacobi sweeps, omega 0.8, before and
-// after; the one-node grid exactly) on a grid of nx x nx nodes; st: the
-// stencils of this grid and of all below it. Column by column, in FP64.
-static std::vector<double> vcycle_matrix(int nx, const std::vector<std::vector<double>>& st) {
-  const int n = nx * nx;
-  std::vector<double> M((size_t)n * n);
-  std::function<std::vector<double>(size_t, int, const std::vector<double>&)> cycle =
-      [&](size_t g, int m, const std::vector<double>& b) {
-        const auto& s9 = st[g];
-        auto at = [&](const std::vector<double>& v, int x, int y, int w) {
-          return x < 0 || y < 0 || x >= w || y >= w ? 0.0 : v[y * w + x];
-        };
-        auto residual = [&](const std::vector<double>& x) {
-          std::vector<double> r(b);
-          for (int i = 0; i < m * m; ++i)
-            for (int e = 0; e < 9; ++e) r[i] -= s9[i * 9 + e] * at(x, i % m + e % 3 - 1, i / m + e / 3 - 1, m);
-          return r;
-        };
-        std::vector<double> x(m * m, 0.0);
-        if (m == 1) {
-          x[0] = b[0] / s9[4];
-          return x;
-        }
-        auto sweep = [&]() {
-          const auto r = residual(x);
-          for (int i = 0; i < m * m; ++i) x[i] += 0.8 / s9[i * 9 + 4] * r[i];
-        };
-        for (int k = 0; k < 2; ++k) sweep();
-        const auto r = residual(x);
-        const int mc = (m - 1) / 2;
-        std::vector<double> bc(mc * mc, 0.0);
-        auto weight = [](int d) { return d == 0 ? 1.0 : 0.5; };
-        for (int c = 0; c < mc * mc; ++c)
-          for (int e = 0; e < 9; ++e)
-            bc[c] += weight(e % 3 - 1) * weight(e / 3 - 1) * at(r, 2 * (c % mc) + e % 3, 2 * (c / mc) + e / 3, m);
-        const auto xc = cycle(g + 1, mc, bc);
-        for (int c = 0; c < mc * mc; ++c)
-          for (int e = 0; e < 9; ++e)
-            x[(2 * (c / mc) + e / 3) * m + 2 * (c % mc) + e % 3] += weight(e % 3 - 1) * weight(e / 3 - 1) * xc[c];
-        for (int k = 0; k < 2; ++k) sweep();
-        return x;
-      };
-  for (int j = 0; j < n; ++j) {
-    std::vector<double> b(n, 0.0);
-    b[j] = 1.0;
-    const auto x = cycle(0, nx, b);
-    for (int i = 0; i < n; ++i) M[(size_t)i * n + j] = x[i];
+// after; the one-node grid exactly) on a grid of m x m nodes; st: the stencils
+// of this grid and of those below it. In FP64, for all unit right-hand sides at
+// once: vectors are [m m][N] with N columns.
+static std::vector<double> vcycle_columns(const std::vector<double>* st, int m, int N, const std::vector<double>& b) {
+  const int n = m * m;
+  const std::vector<double>& s9 = *st;
+  std::vector<double> x((size_t)n * N, 0.0), r(b);
+  auto add = [N](double* to, double a, const double* from) {
+    for (int j = 0; j < N; ++j) to[j] += a * from[j];
+  };
+  if (m == 1) {
+    add(x.data(), 1.0 / s9[4], b.data());
+    return x;
   }
-  return M;
+  auto residual = [&]() {
+    r = b;
+    for (int i = 0; i < n; ++i)
+      for (int e = 0; e < 9; ++e) {
+        const int X = i % m + e % 3 - 1, Y = i / m + e / 3 - 1;
+        if (X >= 0 && Y >= 0 && X < m && Y < m) add(&r[(size_t)i * N], -s9[i * 9 + e], &x[(size_t)(Y * m + X) * N]);
+      }
+  };
+  auto sweep = [&]() {   // r is the residual of x on entry
+    for (int i = 0; i < n; ++i) add(&x[(size_t)i * N], 0.8 / s9[i * 9 + 4], &r[(size_t)i * N]);
+    residual();
+  };
+  sweep();
+  sweep();
+  const int mc = (m - 1) / 2;
+  auto transfer = [&](auto f) {   // f(coarse node, fine node, weight)
+    for (int c = 0; c < mc * mc; ++c)
+      for (int e = 0; e < 9; ++e)
+        f(c, (2 * (c / mc) + e / 3) * m + 2 * (c % mc) + e % 3, (e % 3 == 1 ? 1.0 : 0.5) * (e / 3 == 1 ? 1.0 : 0.5));
+  };
+  std::vector<double> bc((size_t)mc * mc * N, 0.0);
+  transfer([&](int c, int i, double w) { add(&bc[(size_t)c * N], w, &r[(size_t)i * N]); });
+  const std::vector<double> xc = vcycle_columns(st + 1, mc, N, bc);
+  transfer([&](int c, int i, double w) { add(&x[(size_t)i * N], w, &xc[(size_t)c * N]); });
+  residual();
+  sweep();
+  sweep();
+  return x;
+}
+
+static std::vector<double> vcycle_matrix(int m, const std::vector<std::vector<double>>& st) {
+  const int n = m * m;
+  std::vector<double> unit((size_t)n * n, 0.0);
+  for (int i = 0; i < n; ++i) unit[(size_t)i * n + i] = 1.0;
+  return vcycle_columns(st.data(), m, n, unit);
 }
 
 static int upload_grid(GridLevel& g, const std::vector<double>& st, bool finest) {
