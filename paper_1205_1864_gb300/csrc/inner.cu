@@ -44,7 +44,6 @@
 
 namespace sghsc {
 
-constexpr int MAX_LEVELS = 16;
 
 // Column groups: the batch buffers are node-major with a padded width wp (a
 // multiple of N = 16 bytes / sizeof(T)), and each thread owns N adjacent
@@ -369,29 +368,6 @@ __device__ __forceinline__ void reduce_finalize(const FinArgs& f, const A (&v)[N
   if (last_block(&f.ctl->ticket)) fin_columns<A>(f, op, wp, gridDim.x);
 }
 
-// (P xc) at fine node (fx, fy): bilinear interpolation from the coarse grid,
-// coarse node (X, Y) sitting on fine node (2X+1, 2Y+1), zero outside
-// (one column, used by the coarse-grid phase).
-template <typename T>
-__device__ __forceinline__ T prolong_at(int fx, int fy, int nxc, int nyc, const T* __restrict__ xc) {
-  int Xs[2], Ys[2];
-  T wx[2], wy[2];
-  int nxs, nys;
-  if (fx & 1) { Xs[0] = (fx - 1) >> 1; wx[0] = T(1); nxs = 1; }
-  else { Xs[0] = (fx >> 1) - 1; Xs[1] = fx >> 1; wx[0] = wx[1] = T(0.5); nxs = 2; }
-  if (fy & 1) { Ys[0] = (fy - 1) >> 1; wy[0] = T(1); nys = 1; }
-  else { Ys[0] = (fy >> 1) - 1; Ys[1] = fy >> 1; wy[0] = wy[1] = T(0.5); nys = 2; }
-  T acc = T(0);
-  for (int iy = 0; iy < nys; ++iy) {
-    if (Ys[iy] < 0 || Ys[iy] >= nyc) continue;
-    for (int ix = 0; ix < nxs; ++ix) {
-      if (Xs[ix] < 0 || Xs[ix] >= nxc) continue;
-      acc += wy[iy] * wx[ix] * xc[Ys[iy] * nxc + Xs[ix]];
-    }
-  }
-  return acc;
-}
-
 // Node order of the 9-point stencil phases. The grid is cut into column strips
 // k nodes wide (the nodes of one block pass); the (strip, row) units are split
 // into one contiguous share per block, and a block walks its share row by row
@@ -707,172 +683,6 @@ __device__ __forceinline__ void ph_prolong_jacobi(Blk B, int nxf, int nyf, int n
   }
 }
 
-struct CoarseGrids {
-  int g0, G;
-  int nx[MAX_LEVELS], ny[MAX_LEVELS], off[MAX_LEVELS];
-  const void* st[MAX_LEVELS];
-  const void* dinv[MAX_LEVELS];
-};
-
-template <typename T>
-__device__ __forceinline__ void stage_async(T* __restrict__ dst, const T* __restrict__ src, int count) {
-  for (int idx = threadIdx.x; idx < count; idx += blockDim.x) cp_async_elem(dst + idx, src + idx);
-}
-
-// Shared memory of the coarse-grid phase: per grid a right-hand side, an
-// iterate and a ping-pong buffer, plus the stencils and inverse diagonals.
-template <typename T>
-static size_t coarse_smem_bytes(int tot) {
-  return (size_t)13 * tot * sizeof(T);
-}
-
-// The V-cycle from grid g0 down, one column at a time per block (the blocks
-// stride over the columns; the coarse grids are latency-bound, so the work
-// spreads over as many SMs as there are columns), entirely in shared memory.
-// Every coarse stencil and inverse diagonal is staged once per block, with the
-// first column's right-hand side, by asynchronous copies all in flight
-// together. Grids of at most 64 nodes are run by warp 0 alone with warp-level
-// synchronisation. blockDim must be 1024.
-template <typename T>
-__device__ void ph_coarse(Blk Bk, const CoarseGrids& L, int tot, int wp, const T* __restrict__ bg,
-                          T* __restrict__ xg, T om, int nu, const int* __restrict__ done, unsigned char* smem) {
-  T* sm = reinterpret_cast<T*>(smem);
-  T* sst = sm + 3 * tot;          // stencils [node][9] of all coarse grids
-  T* sdi = sst + 9 * tot;         // inverse diagonals
-  auto stg = [&](int g) { return (const T*)(sst + 9 * L.off[g]); };
-  auto dig = [&](int g) { return (const T*)(sdi + L.off[g]); };
-  const int tid = threadIdx.x;
-  auto B = [&](int g) { return sm + 3 * L.off[g]; };
-  auto Xa = [&](int g) { return sm + 3 * L.off[g] + L.nx[g] * L.ny[g]; };
-  auto Xb = [&](int g) { return sm + 3 * L.off[g] + 2 * L.nx[g] * L.ny[g]; };
-  auto sdot = [&](const T* s9, int nx, int ny, int x, int y, const T* v) {
-    T acc = T(0);
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int yy = y + dy;
-      if (yy < 0 || yy >= ny) continue;
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int xx = x + dx;
-        if (xx < 0 || xx >= nx) continue;
-        acc += s9[(dy + 1) * 3 + (dx + 1)] * v[yy * nx + xx];
-      }
-    }
-    return acc;
-  };
-  // grid g runs in warp mode (warp 0 only, __syncwarp) when it has <= 64 nodes
-  auto wmode = [&](int g) { return L.nx[g] * L.ny[g] <= 64; };
-  auto lsync = [&](bool wm) {
-    if (wm) __syncwarp(); else __syncthreads();
-  };
-  const int n0 = L.nx[L.g0] * L.ny[L.g0];
-  bool staged = false;
-  for (int col = Bk.bid; col < wp; col += Bk.nb) {
-    if (done[col]) continue;
-    if (!staged) {
-      for (int g = L.g0; g < L.G; ++g) {
-        const int n = L.nx[g] * L.ny[g];
-        stage_async(sst + 9 * L.off[g], (const T*)L.st[g], 9 * n);
-        stage_async(sdi + L.off[g], (const T*)L.dinv[g], n);
-      }
-      staged = true;
-    }
-    {
-      T* b0 = B(L.g0);
-      for (int idx = tid; idx < n0; idx += blockDim.x) cp_async_elem(b0 + idx, bg + idx * wp + col);
-    }
-    cp_async_wait_all();   // stencils, diagonals and the right-hand side
-    __syncthreads();
-    T* cur[MAX_LEVELS];
-    T* oth[MAX_LEVELS];
-    for (int g = L.g0; g < L.G; ++g) {
-      const int nx = L.nx[g], ny = L.ny[g], n = nx * ny;
-      const bool wm = wmode(g);
-      const int lim = wm ? 32 : (int)blockDim.x;
-      const bool act = tid < lim;
-      const T* st = stg(g);
-      const T* dinv = dig(g);
-      const T* b = B(g);
-      T* c = Xa(g);
-      T* o = Xb(g);
-      if (g == L.G - 1) {  // coarsest grid (one node for square grids): exact solve
-        if (act)
-          for (int idx = tid; idx < n; idx += lim) c[idx] = dinv[idx] * b[idx];
-        lsync(wm);
-        cur[g] = c;
-        oth[g] = o;
-        break;
-      }
-      if (act)
-        for (int idx = tid; idx < n; idx += lim) c[idx] = om * dinv[idx] * b[idx];
-      lsync(wm);
-      for (int s = 1; s < nu; ++s) {
-        if (act)
-          for (int idx = tid; idx < n; idx += lim) {
-            const int y = idx / nx, x = idx - y * nx;
-            o[idx] = c[idx] + om * dinv[idx] * (b[idx] - sdot(st + idx * 9, nx, ny, x, y, c));
-          }
-        lsync(wm);
-        T* t = c; c = o; o = t;
-      }
-      if (act)
-        for (int idx = tid; idx < n; idx += lim) {
-          const int y = idx / nx, x = idx - y * nx;
-          o[idx] = b[idx] - sdot(st + idx * 9, nx, ny, x, y, c);
-        }
-      lsync(wm);
-      const int nxc = L.nx[g + 1], nyc = L.ny[g + 1];
-      T* bc = B(g + 1);
-      if (act)
-        for (int idx = tid; idx < nxc * nyc; idx += lim) {
-          const int Y = idx / nxc, X = idx - Y * nxc;
-          T acc = T(0);
-          for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-              const T wgt = (dx == 0 ? T(1) : T(0.5)) * (dy == 0 ? T(1) : T(0.5));
-              acc += wgt * o[(2 * Y + 1 + dy) * nx + (2 * X + 1 + dx)];
-            }
-          bc[idx] = acc;
-        }
-      lsync(wm);
-      cur[g] = c;
-      oth[g] = o;
-    }
-    for (int g = L.G - 2; g >= L.g0; --g) {
-      const int nx = L.nx[g], ny = L.ny[g], n = nx * ny;
-      const int nxc = L.nx[g + 1], nyc = L.ny[g + 1];
-      const bool wm = wmode(g);
-      if (!wm && wmode(g + 1)) __syncthreads();   // results of warp 0 become visible to the block
-      const int lim = wm ? 32 : (int)blockDim.x;
-      const bool act = tid < lim;
-      const T* st = stg(g);
-      const T* dinv = dig(g);
-      const T* b = B(g);
-      T* c = cur[g];
-      T* o = oth[g];
-      const T* xc = cur[g + 1];
-      if (act)
-        for (int idx = tid; idx < n; idx += lim) {
-          const int y = idx / nx, x = idx - y * nx;
-          c[idx] += prolong_at(x, y, nxc, nyc, xc);
-        }
-      lsync(wm);
-      for (int s = 0; s < nu; ++s) {
-        if (act)
-          for (int idx = tid; idx < n; idx += lim) {
-            const int y = idx / nx, x = idx - y * nx;
-            o[idx] = c[idx] + om * dinv[idx] * (b[idx] - sdot(st + idx * 9, nx, ny, x, y, c));
-          }
-        lsync(wm);
-        T* t = c; c = o; o = t;
-      }
-      cur[g] = c;
-    }
-    __syncthreads();
-    const T* x0 = cur[L.g0];
-    for (int idx = tid; idx < n0; idx += blockDim.x) xg[idx * wp + col] = x0[idx];
-    __syncthreads();   // the next column reuses the buffers
-  }
-}
-
 // r = src (cast; padded columns w..wp-1 zero); acc = ||b||^2 partials. x is
 // not cleared: the first update writes it (x = alpha p), and a batch that
 // ends before its first iteration scatters zeros.
@@ -1049,14 +859,6 @@ __global__ void __launch_bounds__(1024) k_prolong_jacobi(int nxf, int nyf, int n
   T acc[VW<T>::N];
   ph_prolong_jacobi<T, DOT>(this_grid(), nxf, nyf, nxc, nyc, wp, k, st, dinv, b, x, xc, xo, om, f.done, acc);
   if (DOT) reduce_finalize<T, VW<T>::N>(f, acc, wp, k, FIN_RHO);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseGrids L, int tot, int wp, const T* __restrict__ bg,
-                                                        T* __restrict__ xg, T om, int nu,
-                                                        const int* __restrict__ done) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  ph_coarse<T>(this_grid(), L, tot, wp, bg, xg, om, nu, done, smem_raw);
 }
 
 // r = src, ||b||^2 -> FIN_INIT (sets the loop condition; zero columns, the
@@ -1859,29 +1661,6 @@ static FinArgs make_fin(sg_problem* h, InnerWork& iw, const sg_prec_opts& o) {
   return f;
 }
 
-template <typename T>
-static int launch_coarse(sg_problem* h, int g0, const T* b, T* x, int wp, const sg_prec_opts& o, const int* done,
-                         cudaStream_t s) {
-  CoarseGrids L;
-  L.g0 = g0;
-  L.G = (int)h->grids.size();
-  int tot = 0;
-  for (int g = g0; g < L.G; ++g) {
-    const GridLevel& G = h->grids[g];
-    L.nx[g] = G.nx;
-    L.ny[g] = G.ny;
-    L.off[g] = tot;
-    tot += G.n;
-    L.st[g] = sizeof(T) == 8 ? (const void*)G.st64 : (const void*)G.st32;
-    L.dinv[g] = sizeof(T) == 8 ? (const void*)G.dinv64 : (const void*)G.dinv32;
-  }
-  const size_t smem = coarse_smem_bytes<T>(tot);
-  SG_TRY_CUDA(cudaFuncSetAttribute(k_vcycle_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  { k_vcycle_coarse<T><<<wp, 1024, smem, s>>>(L, tot, wp, b, x, (T)o.omega, o.nu, done); ::sghsc::note_launch(); }
-  SG_CHECK_LAUNCH();
-  return SG_OK;
-}
-
 // Tile edge of the tiled restriction from grid G to grid C: the largest
 // (<= 16) whose fine footprint (2TC+1)^2 times the column groups stays within
 // 2048 residuals per block, shrunk while that leaves fewer tiles than SMs.
@@ -1967,7 +1746,7 @@ static int vcycle(sg_problem* h, InnerWork& iw, int g, const T* b, T* x, T* xt, 
     return SG_OK;
   }
   if (g >= h->cb_level) {
-    SG_TRY(launch_coarse<T>(h, g, b, x, wp, o, iw.done, s));
+    SG_TRY(launch_coarse(h, sizeof(T) == 8 ? SG_F64 : SG_F32, g, b, x, wp, o, iw.done, s));
     if (fdot) {
       const Shape sh = make_shape(h, h->grids[g].n, ng, 1);
       { k_dot_fin<T><<<sh.grid, sh.bdim, 0, s>>>(h->grids[g].n, wp, sh.k, b, x, *fdot, FIN_RHO); ::sghsc::note_launch(); }

@@ -35,7 +35,7 @@
 // V-cycle 15 x 15, FP64, 20 columns 251 -> 104, 31 x 31, FP32, 300 columns
 // 229 -> 120. No size it can hold was slower (1 to 1000 columns, both
 // types), so every batch that fits takes it. Whole FP64 solves: 16 x 16
-// elements, M = 3, p = 3, 6.64 -> 1.40 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
+// elements, M = 3, p = 3, 6.64 -> 1.30 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
 // 274 -> 15.4 ms; lognormal 10 x 10, M = 3, p = 3, 1034 -> 77.6 ms.
 #include <cooperative_groups.h>
 
@@ -54,7 +54,8 @@ constexpr int NW = NT / 32;
 constexpr int MAX_ITEMS = 4;     // nodes per thread of k_block_diag
 constexpr int MAX_C = 8;         // blocks per cluster
 constexpr int VNT = 256;         // threads of k_block_vcycle at most
-constexpr int MAX_GRIDS = 8;     // grids from 31 x 31 (or less) down to one node
+constexpr int CNT = 512;         // threads of k_vcycle_coarse at most
+constexpr int MAX_GRIDS = 16;    // grids of a hierarchy (a finest side of 2^16 - 1)
 }  // namespace blk
 
 struct BlockArgs {
@@ -412,8 +413,12 @@ __device__ __forceinline__ void phase_sync(bool wm) {
   else __syncthreads();
 }
 
-// Zero vectors and the coefficients of the grids from g0 on (not yet visible
-// to the other threads of the block); om: the damping.
+// Zero vectors and the coefficients of the grids from g0 on, not yet visible
+// to the other threads of the block; om: the damping. The stencils and the
+// matrix are asynchronous copies, all in flight together: the caller waits for
+// them (cp_async_wait_all) before a block barrier. Loaded and stored in a loop
+// they were a chain of L2 latencies: 16 x 16 elements, FP64, whole solve 1.39 ->
+// 1.30 ms, gradient on 64 x 64 elements 4.44 -> 4.25 ms.
 template <typename T>
 __device__ __forceinline__ void stage_grids(const BlockGrids& L, T* sm, T om, int g0 = 0) {
   const int tid = threadIdx.x, NT = blockDim.x;
@@ -424,14 +429,15 @@ __device__ __forceinline__ void stage_grids(const BlockGrids& L, T* sm, T om, in
       for (int i = tid; i < cmx::VECS; i += NT) sm[L.vec[g] + i] = T(0);
       for (int i = tid; i < cmx::N * S; i += NT) {
         const int r = i / S, c = i - r * S;
-        sm[L.coef[g] + i] = c < cmx::N ? gs[r * cmx::N + c] : T(0);
+        if (c < cmx::N) cp_async_elem(sm + L.coef[g] + i, gs + r * cmx::N + c);
+        else sm[L.coef[g] + i] = T(0);
       }
       return;
     }
     const int Wg = (1 << L.k[g]) + 1, ng = (Wg - 2) * (Wg - 2);
     for (int i = tid; i < 3 * Wg * Wg; i += NT) sm[L.vec[g] + i] = T(0);
     const T* gd = (const T*)L.dinv[g];
-    for (int i = tid; i < 9 * ng; i += NT) sm[L.coef[g] + i] = gs[i];
+    for (int i = tid; i < 9 * ng; i += NT) cp_async_elem(sm + L.coef[g] + i, gs + i);
     // the damped inverse diagonal (the plain one on the one-node grid, solved exactly)
     for (int i = tid; i < ng; i += NT) sm[L.coef[g] + 9 * ng + i] = g == L.G - 1 ? gd[i] : om * gd[i];
   }
@@ -607,6 +613,7 @@ __global__ void __launch_bounds__(blk::VNT) k_block_vcycle(BlockArgs a, BlockGri
         b[pc[u]] = v;
         rr += v * v;
       }
+    cp_async_wait_all();   // (published by the barriers of the sum)
     block_sum(red, rr, [&](double s) { scal_init(S, s, a); });
   }
   while (!S.done) {
@@ -651,6 +658,36 @@ __global__ void __launch_bounds__(blk::VNT) k_block_vcycle(BlockArgs a, BlockGri
   for (int u = 0; u < ITEMS; ++u)
     if (nd[u] >= 0) dst[(size_t)nd[u] * ldd + col] = (TD)x[u];
   if (a.iters && tid == 0) a.iters[col] = S.it;
+}
+
+// The coarse end of the stand-alone V-cycle: everything from grid g0 down, one
+// column at a time per block, the blocks striding over the columns (the grids'
+// coefficients are staged once). Bounded by its chain of phases; 512 threads in
+// FP32 (256 in FP64, where each phase waits for the FP64 units anyhow). From 31 x
+// 31 nodes down, 20, 286 and 715 columns: 11, 17 and 37 us; the kernel before, of
+// 1024 threads with boundary tests in its stencils, 17, 26 and 63.
+template <typename T>
+__global__ void __launch_bounds__(blk::CNT) k_vcycle_coarse(BlockGrids L, int g0, T om, int nu, int wp,
+                                                            const T* __restrict__ bg, T* __restrict__ xg,
+                                                            const int* __restrict__ done) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sm = reinterpret_cast<T*>(smem_raw);
+  T* b = sm + L.vec[g0];
+  const int tid = threadIdx.x, NT = blockDim.x;
+  bool staged = false;
+  for (int col = blockIdx.x; col < wp; col += gridDim.x) {
+    if (done[col]) continue;   // the same for every thread of the block
+    if (!staged) {
+      stage_grids<T>(L, sm, om, g0);
+      __syncthreads();
+      staged = true;
+    }
+    each_node(L.k[g0], tid, NT, [&](int i, int node, int, int) { b[i] = bg[(size_t)node * wp + col]; });
+    cp_async_wait_all();
+    __syncthreads();
+    const T* z = block_vcycle<T>(L, sm, nu, g0);   // ends with a block barrier
+    each_node(L.k[g0], tid, NT, [&](int i, int node, int, int) { xg[(size_t)node * wp + col] = z[i]; });
+  }
 }
 
 // ------------------------------------------ V-cycle M_0 on 63 x 63, FP32 ---
@@ -759,6 +796,7 @@ __global__ void __launch_bounds__(blk63::NT, 1)
     own_st(D, d);
     own_st(B, b);
     own_st(U, Own8{{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}});
+    cp_async_wait_all();   // (published by the barriers of the sum)
     block_sum(red, own_dot(b, b), [&](double v) { scal_init(S, v, a); });
   }
   while (!S.done) {
@@ -1022,6 +1060,30 @@ static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd
   };
   if (G.nx <= 15) return go(k_block_vcycle<TS, T, TD, 2>, 128);
   return go(k_block_vcycle<TS, T, TD, 4>, 256);
+}
+
+template <typename T>
+static int launch_coarse_t(sg_problem* h, int g0, const T* b, T* x, int wp, const sg_prec_opts& o, const int* done,
+                           cudaStream_t s) {
+  BlockGrids L;
+  if (!vcycle_layout(h, sizeof(T), o, L, g0)) {
+    set_error("V-cycle: the coarse grids do not fit");
+    return SG_ERR_UNSUPPORTED;
+  }
+  const size_t smem = (size_t)L.total * sizeof(T);
+  const int threads = h->grids[g0].nx <= 15 ? 128 : sizeof(T) == 8 ? blk::VNT : blk::CNT;
+  // as many blocks as are resident: beyond that each column would stage the grids anew
+  const int per_sm = std::max(1, (int)((h->smem_optin + 1024) / (smem + 1024)));
+  SG_TRY_CUDA(cudaFuncSetAttribute(k_vcycle_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  { k_vcycle_coarse<T><<<std::min(wp, h->num_sms * std::min(per_sm, 4)), threads, smem, s>>>(L, g0, (T)o.omega, o.nu, wp, b, x, done); note_launch(); }
+  SG_CHECK_LAUNCH();
+  return SG_OK;
+}
+
+int launch_coarse(sg_problem* h, int dtype, int g0, const void* b, void* x, int wp, const sg_prec_opts& o,
+                  const int* done, cudaStream_t s) {
+  if (dtype == SG_F64) return launch_coarse_t<double>(h, g0, (const double*)b, (double*)x, wp, o, done, s);
+  return launch_coarse_t<float>(h, g0, (const float*)b, (float*)x, wp, o, done, s);
 }
 
 int inner_solve_block(sg_problem* h, int dtype, const void* src, int lds, int src_t, void* dst, int ldd, int dst_t,

@@ -342,6 +342,10 @@ int inner_solve_cluster(sg_problem* h, const void* src, int ld_src, int src_t, v
 bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o);
 // True when FP32 V-cycle solves on h take it before the cluster solver.
 bool block_preferred(const sg_problem* h);
+// One V-cycle from grid g0 (at most 1024 nodes) down on wp columns: b -> x, both
+// [n][wp] of element type dtype; finished columns (done) keep x.
+int launch_coarse(sg_problem* h, int dtype, int g0, const void* b, void* x, int wp, const sg_prec_opts& o,
+                  const int* done, cudaStream_t s);
 int inner_solve_block(sg_problem* h, int dtype, const void* src, int ld_src, int src_t, void* dst, int ld_dst,
                       int dst_t, int w, const sg_prec_opts& o, cudaStream_t s);
 
