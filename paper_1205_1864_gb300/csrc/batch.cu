@@ -371,9 +371,16 @@ int sg_autotune(sg_problem* h, void* stream) {
     }
   }
   SG_TRY(autotune_k1(h, SG_F64, (cudaStream_t)stream));
-  // the FP32 full product takes the row kernel (fixed shape) where it applies
-  // (up to 511 columns the row kernel has no shape to tune either, but the general kernel's is still reported)
-  if (h->P < 512 || !rows32_usable(h, h->all, h->P, true)) SG_TRY(autotune_k1(h, SG_F32, (cudaStream_t)stream));
+  // the FP32 full product takes the row kernel (fixed shape) where it applies; up
+  // to 511 columns the general kernel's shape is still tuned and reported, so it
+  // is the general kernel that is timed
+  if (h->P < 512 || !rows32_usable(h, h->all, h->P, true)) {
+    const int staged = h->staged_pairs;
+    h->staged_pairs = 0;
+    const int r = autotune_k1(h, SG_F32, (cudaStream_t)stream);
+    h->staged_pairs = staged;
+    SG_TRY(r);
+  }
   SG_TRY(autotune_outer(h, (cudaStream_t)stream, false));
   // the double-float pair-form kernel has a fixed shape; tune the general one only when it stands in
   if (!df_pairs_usable(h, h->all, h->P)) SG_TRY(autotune_outer(h, (cudaStream_t)stream, true));
