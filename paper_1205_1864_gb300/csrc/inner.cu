@@ -766,6 +766,78 @@ __device__ __forceinline__ void ph_matvec_p(Blk B, int nx, int ny, int wp, int k
   }
 }
 
+// The same, a thread walking down its strip with the sums of three rows in
+// registers: the three values of a row complete the sum of the row above,
+// continue its own and start the one below (stencil9's order), so z and p_old
+// are read three times each and not nine; a share reads one row more at either
+// end. Bounded by memory and, in narrow batches, by latency. FP32, 20 and 715
+// columns on 255 x 255 nodes, 715 on 511 x 511: 17, 180 and 757 us node by node,
+// 15, 154 and 646 by rows.
+template <typename T>
+__device__ __forceinline__ void ph_matvec_p_rows(Blk B, int nx, int ny, int wp, int k, const T* __restrict__ st,
+                                                 const T* __restrict__ z, const T* __restrict__ pold,
+                                                 T* __restrict__ pnew, T* __restrict__ q, bool first,
+                                                 const T* __restrict__ beta, const int* __restrict__ done,
+                                                 T (&acc)[VW<T>::N]) {
+  constexpr int N = VW<T>::N;
+#pragma unroll
+  for (int u = 0; u < N; ++u) acc[u] = T(0);
+  int cg, lx;
+  if (!strip_pos(wp / N, k, cg, lx)) return;
+  const int c0 = cg * N;
+  if (done_mask<N>(done, c0) == (1u << N) - 1) return;
+  T bt[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) bt[u] = beta[c0 + u];
+  auto pv = [&](int e, bool in) {
+    Vec<T> v = in ? vld(z + e) : vzero<T>();
+    if (!first && in) {
+      const Vec<T> po = vld(pold + e);
+#pragma unroll
+      for (int u = 0; u < N; ++u) v.a[u] += bt[u] * po.a[u];
+    }
+    return v;
+  };
+  auto add3 = [&](Vec<T>& s, const T* a, const Vec<T>& v0, const Vec<T>& v1, const Vec<T>& v2) {
+    const T a0 = a[0], a1 = a[1], a2 = a[2];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      s.a[u] += a0 * v0.a[u];
+      s.a[u] += a1 * v1.a[u];
+      s.a[u] += a2 * v2.a[u];
+    }
+  };
+  const long long tot = (long long)((nx + k - 1) / k) * ny;
+  int u = (int)(tot * B.bid / B.nb);
+  const int u1 = (int)(tot * (B.bid + 1) / B.nb);
+  while (u < u1) {   // a run of rows ya .. yb - 1 of one strip
+    const int cx = u / ny, ya = u - cx * ny, yb = min(ny, ya + (u1 - u)), x = cx * k + lx;
+    u += yb - ya;
+    if (x >= nx) continue;
+    const bool l = x > 0, r = x < nx - 1;
+    Vec<T> s0 = vzero<T>(), s1 = vzero<T>(), pc = vzero<T>();   // sums of rows t - 1 and t, p on row t - 1
+    for (int t = ya - 1; t <= yb; ++t) {
+      const bool in = t >= 0 && t < ny;
+      const int node = t * nx + x, i = in ? node * wp + c0 : 0;
+      const Vec<T> v0 = pv(i - wp, in && l), v1 = pv(i, in), v2 = pv(i + wp, in && r);
+      if (t > ya) {
+        add3(s0, st + (node - nx) * 9 + 6, v0, v1, v2);
+        const int o = (node - nx) * wp + c0;
+        vst(pnew + o, pc);
+        vst(q + o, s0);
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc[e] += pc.a[e] * s0.a[e];
+      }
+      Vec<T> s2 = vzero<T>();
+      if (t >= ya && t < yb) add3(s1, st + node * 9 + 3, v0, v1, v2);
+      if (t + 1 < yb) add3(s2, st + (node + nx) * 9, v0, v1, v2);
+      s0 = s1;
+      s1 = s2;
+      pc = v1;
+    }
+  }
+}
+
 // x += alpha p_new; r -= alpha q; acc = r . r. Finished columns keep x and r.
 template <typename T>
 __device__ __forceinline__ void ph_update_xr(Blk B, int n, int wp, int k, const T* __restrict__ pnew,
@@ -943,6 +1015,17 @@ __global__ void __launch_bounds__(1024) k_matvec_p(int nx, int ny, int wp, int k
   T acc[VW<T>::N];
   ph_matvec_p<T>(this_grid(), nx, ny, wp, k, st, z, (it & 1) ? pB : pA, (it & 1) ? pA : pB, q, it == 0,
                  beta_of<T>(f), f.done, acc);
+  reduce_finalize<T, VW<T>::N>(f, acc, wp, k, FIN_ALPHA);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(1024) k_matvec_p_rows(int nx, int ny, int wp, int k, const T* __restrict__ st,
+                                                        const T* __restrict__ z, T* __restrict__ pA,
+                                                        T* __restrict__ pB, T* __restrict__ q, FinArgs f) {
+  const int it = f.ctl->it;
+  T acc[VW<T>::N];
+  ph_matvec_p_rows<T>(this_grid(), nx, ny, wp, k, st, z, (it & 1) ? pB : pA, (it & 1) ? pA : pB, q, it == 0,
+                      beta_of<T>(f), f.done, acc);
   reduce_finalize<T, VW<T>::N>(f, acc, wp, k, FIN_ALPHA);
 }
 
@@ -1861,7 +1944,16 @@ static int inner_solve_t(sg_problem* h, const void* src, int ld_src, int src_t, 
     f.flag = lc.flag;
     const T* z = nullptr;
     SG_TRY(vcycle<T>(h, iw, 0, r, (T*)iw.z, (T*)iw.zt, wp, o, bs, &f, &z));
-    { k_matvec_p<T><<<sh.grid, sh.bdim, 0, bs>>>(G.nx, G.ny, wp, sh.k, st, z, pA, pB, q, f); ::sghsc::note_launch(); }
+    // by rows, but for FP64 shares of less than two rows (127 x 127 nodes, 20
+    // columns: 38 us by rows, 34 node by node; 1 column 24 and 33)
+    bool rows = true;
+    if constexpr (sizeof(T) == 8) {
+      rows = (long long)ceil_div(G.nx, sh.k) * G.ny >= 2LL * sh.grid;
+      if (!rows)
+        { k_matvec_p<<<sh.grid, sh.bdim, 0, bs>>>(G.nx, G.ny, wp, sh.k, st, z, pA, pB, q, f); ::sghsc::note_launch(); }
+    }
+    if (rows)
+      { k_matvec_p_rows<T><<<sh.grid, sh.bdim, 0, bs>>>(G.nx, G.ny, wp, sh.k, st, z, pA, pB, q, f); ::sghsc::note_launch(); }
     { k_update_xr<T><<<sh.grid, sh.bdim, 0, bs>>>(G.n, wp, sh.k, pA, pB, q, x, r, f); ::sghsc::note_launch(); }
     SG_CHECK_LAUNCH();
     return SG_OK;

@@ -50,3 +50,26 @@ def test_inner_solve_with_finished_columns(lib, ne, w):
     ref = krylov.pcg_columns(lambda v: A[0] @ v, B[:, cols].astype(np.float64), lambda r: gmg.vcycle(lv, r), tol=0.0,
                              maxit=2, fixed_iters=2)[0]
     assert np.all(np.abs(X[:, cols] - ref) <= 1e-4 * np.abs(ref).max(axis=0, keepdims=True))
+
+
+@pytest.mark.parametrize("ne,w,prec", [(128, 1, "fp64"), (128, 20, "fp64"), (128, 131, "fp64"), (256, 3, "fp32"),
+                                       (256, 230, "fp32"), (128, 701, "fp32")])
+def test_direction_update_by_rows(lib, ne, w, prec):
+    """The inner CG's p, q = A_0 p kernel walking down its strips (and node by
+    node for FP64 shares of less than two rows: 127 x 127 nodes, 20 columns):
+    shares that begin and end inside a strip, one block's and several strips'.
+    Three steps against the oracle: 1e-10 in FP64, 1e-4 in FP32 (the bars of the
+    solvers at these sizes)."""
+    import torch
+    prob, A, _, _ = problem(ne, 1, 1)
+    h = lib.SGProblem.from_inputs(prob, 1)
+    code, dt, tol = ((lib.SG_F64, torch.float64, 1e-10) if prec == "fp64" else (lib.SG_F32, torch.float32, 1e-4))
+    B = S.random_block(prob.n, w, seed=w).astype(np.float64 if prec == "fp64" else np.float32)
+    X, it = lib.sg_inner_solve(h, torch.tensor(B, dtype=dt, device="cuda"),
+                               lib.prec_opts(precision=code, inner_fixed_iters=3))
+    cols = sorted({0, w // 2, w - 1})
+    lv = gmg.hierarchy(A[0], ne)
+    ref = krylov.pcg_columns(lambda v: A[0] @ v, B[:, cols].astype(np.float64), lambda r: gmg.vcycle(lv, r), tol=0.0,
+                             maxit=3, fixed_iters=3)[0]
+    assert list(it) == [3] * w
+    assert np.abs(X.double().cpu().numpy()[:, cols] - ref).max() <= tol * np.abs(ref).max()
