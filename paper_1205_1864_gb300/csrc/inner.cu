@@ -26,6 +26,8 @@
 //
 // V-cycle kernels (weighted Jacobi, nu sweeps before and after, bilinear
 // transfers, Galerkin coarse operators built in setup.cu):
+//   k_mg_down, k_mg_up  a grid's work in two passes over the batch (mg_fused.cuh;
+//                     FP32, two sweeps, narrow or wide batches); else
 //   k_smooth00        two sweeps from a zero iterate in one pass
 //   k_resid_restrict_t  the residual b - A x formed once per fine node in shared
 //                     memory (tiles of coarse nodes) and restricted
@@ -33,8 +35,10 @@
 //                     first post-smoothing sweep applied to it
 //   k_jacobi          further sweeps; the last sweep of the finest grid also
 //                     reduces r . z for the CG
-//   k_vcycle_coarse   all grids with <= 1024 nodes: one 1024-thread block per column
-//                     runs the rest of the V-cycle in shared memory.
+//   k_vcycle_coarse   all grids with <= 1024 nodes: a block runs the rest of the
+//                     V-cycle of a column in shared memory (inner_block.cu).
+// Grids small enough are solved whole by one block or cluster of blocks per
+// column (inner_block.cu) or by clusters (inner_cluster.cu).
 #include <algorithm>
 #include <mutex>
 

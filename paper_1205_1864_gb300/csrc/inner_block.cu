@@ -18,6 +18,10 @@
 //   k_block_vcycle  M_0 = one V-cycle, finest grid of at most 1024 nodes: one
 //                   block per column, all grids in shared memory with zero
 //                   borders (no boundary tests in the stencils).
+//   k_block_vcycle63  the same on 63 x 63 nodes in FP32, the finest grid's
+//                   stencils in registers.
+//   k_vcycle_coarse  not a solver: the V-cycle's coarse grids for the
+//                   stand-alone kernels, through the same code.
 //
 // What bounds them: the FP64 unit of each SM quarter takes a warp instruction
 // every 69 clocks (measured; one at a time, whatever the number of active
@@ -32,8 +36,8 @@
 // and synchronisation, 20 steps of the diagonal M_0 or 2 of the V-cycle:
 // 29 x 29 nodes, FP64, 20 columns 1412 -> 159 us, 1000 columns 4584 -> 1029;
 // 63 x 63, FP64, 300 columns 2833 -> 1503; 9 x 9, 20 columns 1487 -> 143;
-// V-cycle 15 x 15, FP64, 20 columns 251 -> 104, 31 x 31, FP32, 300 columns
-// 229 -> 120. No size it can hold was slower (1 to 1000 columns, both
+// V-cycle 15 x 15, FP64, 20 columns 251 -> 104 (since then the matrix and the
+// staging below), 31 x 31, FP32, 300 columns 229 -> 120. No size it can hold was slower (1 to 1000 columns, both
 // types), so every batch that fits takes it. Whole FP64 solves: 16 x 16
 // elements, M = 3, p = 3, 6.64 -> 1.30 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
 // 274 -> 15.4 ms; lognormal 10 x 10, M = 3, p = 3, 1034 -> 77.6 ms.
@@ -1041,7 +1045,7 @@ static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd
     if (layout63(h, o, L)) {
       const size_t smem = (blk63::FLOATS + (size_t)L.total) * sizeof(float);
       auto kern = k_block_vcycle63<TS, TD>;
-      SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      SG_TRY(allow_smem(h, kern));
       { kern<<<w, blk63::NT, smem, s>>>(a, L, (float)o.omega, o.nu, G.planes, src, lds, dst, ldd); note_launch(); }
       SG_CHECK_LAUNCH();
       return SG_OK;
@@ -1053,7 +1057,7 @@ static int solve_block_t(sg_problem* h, const TS* src, int lds, TD* dst, int ldd
   }
   const size_t smem = (size_t)L.total * sizeof(T);
   auto go = [&](auto kern, int threads) -> int {
-    SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(allow_smem(h, kern));
     { kern<<<w, threads, smem, s>>>(a, L, (T)o.omega, o.nu, src, lds, dst, ldd); note_launch(); }
     SG_CHECK_LAUNCH();
     return SG_OK;
@@ -1074,7 +1078,7 @@ static int launch_coarse_t(sg_problem* h, int g0, const T* b, T* x, int wp, cons
   const int threads = h->grids[g0].nx <= 15 ? 128 : sizeof(T) == 8 ? blk::VNT : blk::CNT;
   // as many blocks as are resident: beyond that each column would stage the grids anew
   const int per_sm = std::max(1, (int)((h->smem_optin + 1024) / (smem + 1024)));
-  SG_TRY_CUDA(cudaFuncSetAttribute(k_vcycle_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SG_TRY(allow_smem(h, k_vcycle_coarse<T>));
   { k_vcycle_coarse<T><<<std::min(wp, h->num_sms * std::min(per_sm, 4)), threads, smem, s>>>(L, g0, (T)o.omega, o.nu, wp, b, x, done); note_launch(); }
   SG_CHECK_LAUNCH();
   return SG_OK;

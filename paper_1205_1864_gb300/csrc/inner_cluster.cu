@@ -33,7 +33,8 @@
 //
 // Eligibility (cluster_setup): a square hierarchy (power-of-two elements)
 // whose shared-memory plan fits one CTA, at least one cluster resident, FP32.
-// Anything else takes the stand-alone kernels.
+// Grids up to 63 x 63 nodes take the block solvers first (inner_block.cu);
+// anything else the stand-alone kernels.
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -199,7 +199,7 @@ int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, i
   const int rows = E.rows32;
   const size_t smem = rows32_smem(E.ncls, h->nterm, wx, rows);
   auto go = [&](auto kern) -> int {
-    SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(allow_smem(h, kern));
     int per_sm = 0;
     SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
     const int grid = std::min((h->n + rows - 1) / rows, h->num_sms * std::max(per_sm, 1));

@@ -301,6 +301,20 @@ bool rows32_usable(const sg_problem* h, const EdgeList& E, int wx, bool diag);
 int launch_rows32(sg_problem* h, const EdgeList& E, bool diag, const float* X, int ldx, int wx, const float* Yin,
                   int ldyin, float* Y, int ldy, cudaStream_t s);
 
+// Lets a kernel take all the dynamic shared memory a block may have. The limit
+// is an attribute of the function, shared by every handle and thread of the
+// process: set to each launch's own size, one thread could lower it between
+// another's setting and its launch.
+template <typename K>
+inline int allow_smem(const sg_problem* h, K* kern) {
+  cudaFuncAttributes a;
+  SG_TRY_CUDA(cudaFuncGetAttributes(&a, (const void*)kern));
+  const int most = h->smem_optin - (int)a.sharedSizeBytes;
+  if (a.maxDynamicSharedSizeBytes < most)
+    SG_TRY_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  return SG_OK;
+}
+
 // The FP32 stencil copies of a grid (st12, planes) from st32 and dinv32.
 int pack_stencils(GridLevel& g);
 
