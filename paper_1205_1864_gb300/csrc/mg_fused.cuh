@@ -24,7 +24,7 @@
 // stay zero.
 //
 // What bounds it: instruction issue and the block's barrier per row (17 warps on
-// an SM: the rings take its shared memory); DRAM moves 0.4 of its rate. At
+// an SM: the rings take its shared memory); DRAM moves a quarter of its rate. At
 // 255 x 255 x 716 columns the four kernels this replaces took 135 + 180 + 234 +
 // 163 us, these two 150 + 253; a V-cycle 1245 -> 830 us, at 511 x 511
 // 4433 -> 2761 us. Tried: b's own values of five rows in registers (spills at
