@@ -143,7 +143,8 @@ static std::vector<int> block_candidates(int P) {
 
 // Time the full SG product with each candidate block size, in pair and in
 // gather form, and keep the fastest.
-static int autotune_k1(sg_problem* h, int dtype, cudaStream_t s) {
+// whole_warps: the sizes beside the powers of two too.
+static int autotune_k1(sg_problem* h, int dtype, bool whole_warps, cudaStream_t s) {
   const size_t es = dtype == SG_F64 ? 8 : 4;
   const size_t bytes = (size_t)h->n * h->P * es;
   void *X = nullptr, *Y = nullptr;
@@ -157,7 +158,8 @@ static int autotune_k1(sg_problem* h, int dtype, cudaStream_t s) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  const std::vector<int> cands = block_candidates(h->P);
+  std::vector<int> cands = block_candidates(h->P);
+  if (!whole_warps) cands.resize(5);
   const int nc = (int)cands.size();
   int best = 0, best_pairs = 1;
   float best_ms = 1e30f;
@@ -370,14 +372,16 @@ int sg_autotune(sg_problem* h, void* stream) {
       return SG_OK;
     }
   }
-  SG_TRY(autotune_k1(h, SG_F64, (cudaStream_t)stream));
+  SG_TRY(autotune_k1(h, SG_F64, true, (cudaStream_t)stream));
   // the FP32 full product takes the row kernel (fixed shape) where it applies; up
-  // to 511 columns the general kernel's shape is still tuned and reported, so it
-  // is the general kernel that is timed
-  if (h->P < 512 || !rows32_usable(h, h->all, h->P, true)) {
+  // to 511 columns the general kernel's shape is still tuned and reported, for
+  // the forms that the row kernel does not take: it is the general kernel that
+  // is timed, over the powers of two
+  const bool row_kernel = rows32_usable(h, h->all, h->P, true);
+  if (h->P < 512 || !row_kernel) {
     const int staged = h->staged_pairs;
     h->staged_pairs = 0;
-    const int r = autotune_k1(h, SG_F32, (cudaStream_t)stream);
+    const int r = autotune_k1(h, SG_F32, !row_kernel, (cudaStream_t)stream);
     h->staged_pairs = staged;
     SG_TRY(r);
   }
