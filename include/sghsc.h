@@ -355,12 +355,13 @@ int sg_solve_host(sg_problem* h, const double* F_host, double* U_host, const sg_
  * variant, sg_prec_opts.df64), each in two forms, on this problem
  * and keep the fastest for all later calls (products that take a fixed-shape
  * kernel -- the FP32 row kernel, the staged double-float kernel -- are not
- * timed). The forms: the pair form sums each distinct (k, j) of the couplings
+ * timed; below 512 columns the general FP32 kernel still is, for the forms the
+ * row kernel does not take). The forms: the pair form sums each distinct (k, j) of the couplings
  * once per row and keeps those sums in shared memory (fewer multiply-adds);
  * the gather form sums per coupling (no extra shared memory). Where several
  * inner solvers can run a degree level's FP32 batch (grids up to 127 x 127:
- * the stand-alone kernels, the 8- and 16-CTA cluster solvers, the wide one),
- * each is timed on a batch of that width (two fixed PCG iterations) and the
+ * the stand-alone kernels or the block solver, the 8- and 16-CTA cluster
+ * solvers, the wide one), each is timed on a batch of that width (two fixed PCG iterations) and the
  * fastest is kept (sg_inner_path reports it). Allocates temporary blocks and,
  * if absent, the outer solve buffers; invalidates the handle's cached solve
  * graphs. */
