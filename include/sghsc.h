@@ -280,15 +280,15 @@ int sg_inner_solve(sg_problem* h, const void* B, void* X, int w, int dtype,
  * the D_l and A_0 solves inside hsc_precond_apply, mean_precond_apply and
  * sg_solve) run on the cluster-resident solver: one launch per solve, the
  * multigrid hierarchy of each group of 4 columns held in the shared memory of
- * a cluster of 8 thread blocks. 0 when they run on the stand-alone kernels:
- * FP64 solves always do, and so does a grid hierarchy too large for one
+ * a cluster of 8 thread blocks. 0 when they run on the stand-alone kernels or
+ * the block-per-column solver: FP64 solves always do, and so does a grid hierarchy too large for one
  * block's shared memory (finest grids above 127 x 127 nodes), a device that
  * cannot hold such a cluster, or a handle created while the environment
  * variable SGHSC_NO_CLUSTER was 1. A batch of w columns uses the cluster
  * solver only when its ceil(w/4) clusters are all resident at once (on a
- * GB300, up to 60 columns); wider batches take the stand-alone kernels.
- * Grids of 15 x 15, 31 x 31 and 63 x 63 nodes (and smaller ones) take the
- * block-per-column solver first (sg_inner_path). All solvers compute the same method; their results differ by FP32 rounding
+ * GB300, up to 60 columns); wider batches take the block-per-column solver
+ * (grids of 15 x 15, 31 x 31 and 63 x 63 nodes) or the stand-alone kernels.
+ * All solvers compute the same method; their results differ by FP32 rounding
  * (summation order). h NULL: 0. */
 int sg_inner_cluster(const sg_problem* h);
 
@@ -300,10 +300,10 @@ int sg_inner_cluster(const sg_problem* h);
  * 2 the cluster solver with the finest grid in global memory and the coarse
  * grids in shared memory (two blocks per SM, for batches too wide for 1).
  * After sg_autotune, the solver it timed fastest for that width (one of those
- * eligible); else 0 on grids that the block-per-column solver holds (V-cycle:
- * up to 63 x 63 nodes), else the first eligible of 3, 1, 2, then 0. Path 0
- * includes the block-per-column solver (one launch per solve; off on a handle
- * created while SGHSC_NO_BLOCK was 1).
+ * eligible); else the first eligible of 3, 1, then 0 on grids that the
+ * block-per-column solver holds (V-cycle: up to 63 x 63 nodes), 2, then 0.
+ * Path 0 includes the block-per-column solver (one launch per solve; off on a
+ * handle created while SGHSC_NO_BLOCK was 1).
  * h NULL or w <= 0: 0. */
 int sg_inner_path(const sg_problem* h, int w, int dtype);
 

@@ -966,11 +966,12 @@ static bool layout63(const sg_problem* h, const sg_prec_opts& o, BlockGrids& L) 
          vcycle_layout(h, 4, o, L, 1, blk63::FLOATS * sizeof(float));
 }
 
-// FP32 V-cycle solves for which the block solvers are taken before the cluster
-// solver: every grid up to 63 x 63. sg_inner_solve with two steps, clusters and
-// blocks: 15 x 15 nodes 105 and 88 us (20 columns), 238 and 92 (715); 31 x 31
-// 121 and 100, 350 and 165; 63 x 63 134 and 112, 495 and 298. Faster at every
-// width from 1 to 1000, also where a wave of blocks is just begun.
+// FP32 V-cycle solves for which the block solvers are taken before the wide
+// cluster solver: every grid up to 63 x 63. sg_inner_solve with two steps,
+// clusters and blocks: 15 x 15 nodes 100 and 73 us (100 columns); 31 x 31 121
+// and 90; 63 x 63 154 and 107. The on-chip clusters of up to 60 columns come
+// first all the same (cluster_path in inner_cluster.cu): 89 and 75 us, 100 and
+// 87, 112 and 100 (20 columns), what sg_autotune gains there.
 bool block_preferred(const sg_problem* h) {
   if (h->block_off || h->grids.empty()) return false;
   sg_prec_opts o;   // the default smoothing: the larger layout

@@ -33,8 +33,9 @@
 //
 // Eligibility (cluster_setup): a square hierarchy (power-of-two elements)
 // whose shared-memory plan fits one CTA, at least one cluster resident, FP32.
-// Grids up to 63 x 63 nodes take the block solvers first (inner_block.cu);
-// anything else the stand-alone kernels.
+// On grids up to 63 x 63 nodes the block solvers (inner_block.cu) take the
+// batches too wide for the on-chip clusters; anything else takes the
+// stand-alone kernels.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -1325,9 +1326,11 @@ void cluster_free(sg_problem* h) {
 // rows per CTA: the phases of the latency-bound solve are shorter), 1 = the
 // on-chip one with clusters of 8 when all of them are (a second wave would
 // double the solve), 2 = the wide one (finest grid in global memory) when its
-// clusters are, 0 = none of them (the stand-alone kernels).
-// The autotuner's choice for the width (sg_autotune) takes precedence when
-// it is one of the eligible solvers.
+// clusters are and the block solver does not hold the grid, 0 = none of them
+// (the block solver or the stand-alone kernels). The on-chip solvers come
+// before the block solver: that is the order sg_inner_path has always reported.
+// sg_autotune times both, and its choice for the width takes precedence when it
+// is one of the eligible solvers.
 static bool path_eligible(const ClusterSolver* cs, int w, int path) {
   const int ncl = ceil_div(w, 4);
   if (path == 3) return ncl <= cs->maxcl16;
@@ -1341,10 +1344,9 @@ static int cluster_path(const sg_problem* h, int dtype, int w) {
   if (dtype != SG_F32 || !cs) return 0;
   const auto it = h->inner_pick.find(w);
   if (it != h->inner_pick.end() && path_eligible(cs, w, it->second)) return it->second;
-  if (block_preferred(h)) return 0;
-  for (int path : {3, 1, 2})
+  for (int path : {3, 1})
     if (path_eligible(cs, w, path)) return path;
-  return 0;
+  return path_eligible(cs, w, 2) && !block_preferred(h) ? 2 : 0;
 }
 
 std::vector<int> inner_path_candidates(const sg_problem* h, int w) {

@@ -1,0 +1,74 @@
+"""The order in which the inner solvers of small grids are taken, and the
+cluster solvers on the grids that the block-per-column solver holds too
+(``SGHSC_NO_BLOCK=1`` at ``sg_setup`` leaves only them), against the oracle.
+
+Tolerance of the solves: three FP32 steps, 1e-4 of a column's largest entry,
+the bar of the cluster solvers' own tests (about 60 roundings a node and step,
+u = 6e-8, 1e-5, times the spread of A_0's eigenvalues that the V-cycle leaves)."""
+import numpy as np
+import pytest
+
+import sg_inputs as S
+from oracle import gmg, krylov
+from tests.gpu_common import problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import paper_1205_1864_gb300 as L
+    return L
+
+
+@pytest.mark.parametrize("ne", [16, 32, 64, 128])
+def test_on_chip_clusters_come_first(lib, monkeypatch, ne):
+    """A default handle takes the on-chip cluster solver of every batch that
+    one holds, whether or not the block solver holds the grid; the batches
+    beyond go to the block solver (path 0) up to 63 x 63 nodes."""
+    prob, _, _, _ = problem(ne, 1, 1)
+    h = lib.SGProblem.from_inputs(prob, 1)
+    monkeypatch.setenv("SGHSC_NO_BLOCK", "1")
+    c = lib.SGProblem.from_inputs(prob, 1)
+    assert c.inner_path(1) in (1, 3) and c.inner_path(60) == 1
+    for w in (1, 4, 5, 11, 20, 28, 32, 60):
+        assert h.inner_path(w) == c.inner_path(w), w
+    for w in (61, 100, 144):
+        assert c.inner_path(w) == 2 and h.inner_path(w) == (2 if ne == 128 else 0), w
+    assert h.inner_path(400) == 0 and h.inner_path(5, lib.SG_F64) == 0
+
+
+@pytest.mark.parametrize("nu,omega", [(2, 0.8), (1, 0.8), (3, 0.7)])
+@pytest.mark.parametrize("ne,w,path", [(16, 7, 1), (16, 90, 2), (32, 13, 3), (32, 41, 1), (32, 90, 2), (64, 9, 3),
+                                       (64, 41, 1), (64, 90, 2)])
+def test_cluster_solvers_match_oracle(lib, monkeypatch, ne, w, path, nu, omega):
+    import torch
+    prob, A, _, _ = problem(ne, 1, 1)
+    monkeypatch.setenv("SGHSC_NO_BLOCK", "1")
+    h = lib.SGProblem.from_inputs(prob, 1)
+    assert h.inner_path(w) == path
+    lv = gmg.hierarchy(A[0], ne)
+    B = S.random_block(prob.n, w, seed=21 + ne + w).astype(np.float32)
+    B[:, 2] = 0.0
+    X, it = lib.sg_inner_solve(h, torch.tensor(B, device="cuda"), lib.prec_opts(inner_fixed_iters=3, nu=nu, omega=omega))
+    ref, it_ref = krylov.pcg_columns(lambda v: A[0] @ v, B.astype(np.float64),
+                                     lambda r: gmg.vcycle(lv, r, nu=nu, omega=omega), tol=0.0, maxit=3, fixed_iters=3)
+    assert list(it) == list(it_ref)
+    X = X.double().cpu().numpy()
+    assert np.all(np.abs(X - ref) <= 1e-4 * (np.abs(ref).max(axis=0, keepdims=True) + 1e-300))
+    assert np.all(X[:, 2] == 0.0)
+
+
+@pytest.mark.parametrize("ne", [16, 32, 64])
+def test_coarse_matrix_in_the_fp32_block_solver(lib, monkeypatch, ne):
+    """The block solver alone (SGHSC_NO_CLUSTER=1): the 7 x 7 grid and those
+    below as one matrix (the default smoothing) against the grid-by-grid cycle
+    of a damping one rounding away. One step, some 60 roundings a node: 1e-5."""
+    import torch
+    prob, _, _, _ = problem(ne, 1, 1)
+    monkeypatch.setenv("SGHSC_NO_CLUSTER", "1")
+    h = lib.SGProblem.from_inputs(prob, 1)
+    B = torch.tensor(S.random_block(prob.n, 5, seed=ne), dtype=torch.float32, device="cuda")
+    X = [lib.sg_inner_solve(h, B, lib.prec_opts(precision=lib.SG_F32, inner_fixed_iters=1, omega=om))[0]
+         for om in (0.8, float(np.nextafter(0.8, 1)))]
+    assert float((X[0] - X[1]).abs().max()) <= 1e-5 * float(X[1].abs().max())
