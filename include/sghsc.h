@@ -286,8 +286,9 @@ int sg_inner_solve(sg_problem* h, const void* B, void* X, int w, int dtype,
  * cannot hold such a cluster, or a handle created while the environment
  * variable SGHSC_NO_CLUSTER was 1. A batch of w columns uses the cluster
  * solver only when its ceil(w/4) clusters are all resident at once (on a
- * GB300, up to 60 columns); wider batches take the block-per-column solver
- * (grids of 15 x 15, 31 x 31 and 63 x 63 nodes) or the stand-alone kernels.
+ * GB300, up to 60 columns); wider batches, and on grids up to 63 x 63 nodes
+ * those of the preconditioners, take the block-per-column solver or the
+ * stand-alone kernels (sg_inner_path).
  * All solvers compute the same method; their results differ by FP32 rounding
  * (summation order). h NULL: 0. */
 int sg_inner_cluster(const sg_problem* h);
@@ -300,8 +301,10 @@ int sg_inner_cluster(const sg_problem* h);
  * 2 the cluster solver with the finest grid in global memory and the coarse
  * grids in shared memory (two blocks per SM, for batches too wide for 1).
  * After sg_autotune, the solver it timed fastest for that width (one of those
- * eligible); else the first eligible of 3, 1, then 0 on grids that the
- * block-per-column solver holds (V-cycle: up to 63 x 63 nodes), 2, then 0.
+ * eligible); else the first eligible of 3, 1, 2, then 0. On grids that the
+ * block-per-column solver holds (V-cycle: up to 63 x 63 nodes) 0 also for the
+ * widths of the preconditioners' own batches (a degree level's columns, or the
+ * P columns) and for batches too wide for 1.
  * Path 0 includes the block-per-column solver (one launch per solve; off on a
  * handle created while SGHSC_NO_BLOCK was 1).
  * h NULL or w <= 0: 0. */

@@ -966,12 +966,11 @@ static bool layout63(const sg_problem* h, const sg_prec_opts& o, BlockGrids& L) 
          vcycle_layout(h, 4, o, L, 1, blk63::FLOATS * sizeof(float));
 }
 
-// FP32 V-cycle solves for which the block solvers are taken before the wide
-// cluster solver: every grid up to 63 x 63. sg_inner_solve with two steps,
-// clusters and blocks: 15 x 15 nodes 100 and 73 us (100 columns); 31 x 31 121
-// and 90; 63 x 63 154 and 107. The on-chip clusters of up to 60 columns come
-// first all the same (cluster_path in inner_cluster.cu): 89 and 75 us, 100 and
-// 87, 112 and 100 (20 columns), what sg_autotune gains there.
+// FP32 V-cycle solves for which the block solvers are the faster ones: every
+// grid up to 63 x 63. sg_inner_solve with two steps, clusters and blocks: 15 x
+// 15 nodes 89 and 75 us (20 columns), 100 and 73 (100); 31 x 31 100 and 87, 121
+// and 90; 63 x 63 112 and 100, 154 and 107. Which batches take them:
+// cluster_path in inner_cluster.cu.
 bool block_preferred(const sg_problem* h) {
   if (h->block_off || h->grids.empty()) return false;
   sg_prec_opts o;   // the default smoothing: the larger layout

@@ -34,8 +34,8 @@
 // Eligibility (cluster_setup): a square hierarchy (power-of-two elements)
 // whose shared-memory plan fits one CTA, at least one cluster resident, FP32.
 // On grids up to 63 x 63 nodes the block solvers (inner_block.cu) take the
-// batches too wide for the on-chip clusters; anything else takes the
-// stand-alone kernels.
+// preconditioners' own batches and those too wide for the on-chip clusters;
+// anything else takes the stand-alone kernels.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -1327,10 +1327,12 @@ void cluster_free(sg_problem* h) {
 // on-chip one with clusters of 8 when all of them are (a second wave would
 // double the solve), 2 = the wide one (finest grid in global memory) when its
 // clusters are and the block solver does not hold the grid, 0 = none of them
-// (the block solver or the stand-alone kernels). The on-chip solvers come
-// before the block solver: that is the order sg_inner_path has always reported.
-// sg_autotune times both, and its choice for the width takes precedence when it
-// is one of the eligible solvers.
+// (the block solver or the stand-alone kernels). Where the block solver holds
+// the grid it is faster at every width (block_preferred in inner_block.cu), so
+// the preconditioners' own batches take it, tuned or not; for other batches,
+// which only sg_inner_solve sees, the on-chip clusters stay first, the order
+// sg_inner_path has always reported for them. The autotuner's choice for the
+// width takes precedence when it is one of the eligible solvers.
 static bool path_eligible(const ClusterSolver* cs, int w, int path) {
   const int ncl = ceil_div(w, 4);
   if (path == 3) return ncl <= cs->maxcl16;
@@ -1339,14 +1341,27 @@ static bool path_eligible(const ClusterSolver* cs, int w, int path) {
   return path == 0;
 }
 
+// Whether a batch of w columns is one of the preconditioners' own: a degree
+// level's, or the mean-based one's chunks (at most 1024) of the columns of all
+// levels, or of all but the last (the reduced system).
+static bool own_width(const sg_problem* h, int w) {
+  for (int l = 0; l <= h->p; ++l)
+    if (h->off[l + 1] - h->off[l] == w) return true;
+  for (int P : {h->P, h->off[h->p]})
+    if (w == std::min(P, 1024) || w == P % 1024) return true;
+  return false;
+}
+
 static int cluster_path(const sg_problem* h, int dtype, int w) {
   const ClusterSolver* cs = (const ClusterSolver*)h->cl_plan;
   if (dtype != SG_F32 || !cs) return 0;
   const auto it = h->inner_pick.find(w);
   if (it != h->inner_pick.end() && path_eligible(cs, w, it->second)) return it->second;
+  const bool block = block_preferred(h);
+  if (block && own_width(h, w)) return 0;
   for (int path : {3, 1})
     if (path_eligible(cs, w, path)) return path;
-  return path_eligible(cs, w, 2) && !block_preferred(h) ? 2 : 0;
+  return path_eligible(cs, w, 2) && !block ? 2 : 0;
 }
 
 std::vector<int> inner_path_candidates(const sg_problem* h, int w) {

@@ -354,7 +354,7 @@ int inner_solve_cluster(sg_problem* h, const void* src, int ld_src, int src_t, v
 // Any grid that a cluster of blocks holds with the diagonal M_0; with the
 // V-cycle at most 1024 nodes, and 63 x 63 in FP32.
 bool block_usable(const sg_problem* h, int dtype, int w, const sg_prec_opts& o);
-// True when FP32 V-cycle solves on h take it before the wide cluster solver.
+// True when it is the faster solver of FP32 V-cycle solves on h.
 bool block_preferred(const sg_problem* h);
 // One V-cycle from grid g0 (at most 1024 nodes) down on wp columns: b -> x, both
 // [n][wp] of element type dtype; finished columns (done) keep x.

@@ -22,20 +22,70 @@ def lib():
 
 
 @pytest.mark.parametrize("ne", [16, 32, 64, 128])
-def test_on_chip_clusters_come_first(lib, monkeypatch, ne):
-    """A default handle takes the on-chip cluster solver of every batch that
-    one holds, whether or not the block solver holds the grid; the batches
-    beyond go to the block solver (path 0) up to 63 x 63 nodes."""
-    prob, _, _, _ = problem(ne, 1, 1)
-    h = lib.SGProblem.from_inputs(prob, 1)
+def test_order_of_the_solvers(lib, monkeypatch, ne):
+    """Where the block solver holds the grid (up to 63 x 63 nodes) it takes the
+    preconditioners' own batches (degree levels of 1, 3 and 6 columns, 4 and
+    10 in all)
+    and those too wide for the on-chip clusters (path 0); any other batch takes
+    the on-chip cluster solver that holds it."""
+    prob, _, _, _ = problem(ne, 3, 2)
+    h = lib.SGProblem.from_inputs(prob, 2)
     monkeypatch.setenv("SGHSC_NO_BLOCK", "1")
-    c = lib.SGProblem.from_inputs(prob, 1)
+    c = lib.SGProblem.from_inputs(prob, 2)
     assert c.inner_path(1) in (1, 3) and c.inner_path(60) == 1
-    for w in (1, 4, 5, 11, 20, 28, 32, 60):
-        assert h.inner_path(w) == c.inner_path(w), w
+    for w in (1, 3, 4, 6, 10):
+        assert h.inner_path(w) == (c.inner_path(w) if ne == 128 else 0), w
+    for w in (2, 5, 7, 11, 20, 28, 32, 60):
+        assert h.inner_path(w) == c.inner_path(w) != 0, w
     for w in (61, 100, 144):
         assert c.inner_path(w) == 2 and h.inner_path(w) == (2 if ne == 128 else 0), w
     assert h.inner_path(400) == 0 and h.inner_path(5, lib.SG_F64) == 0
+
+
+def _cluster_and_plain(lib, monkeypatch, ne, M, p):
+    """Handles whose inner solves run on the clusters, and on the stand-alone kernels."""
+    prob, A, G, off = problem(ne, M, p)
+    monkeypatch.setenv("SGHSC_NO_BLOCK", "1")
+    c = lib.SGProblem.from_inputs(prob, p)
+    monkeypatch.setenv("SGHSC_NO_CLUSTER", "1")
+    return prob, A, G, off, c, lib.SGProblem.from_inputs(prob, p)
+
+
+@pytest.mark.parametrize("ne,M,p", [(16, 3, 3), (32, 3, 3), (64, 2, 2)])
+def test_algorithm_1_on_clusters(lib, monkeypatch, ne, M, p):
+    """Algorithm 1 with FP32 inner solves of four steps on the clusters: the
+    oracle, and the stand-alone kernels, within 2e-5 of the largest entry (1e-4
+    on 63 x 63 nodes), the bars of these solvers at fixed step counts."""
+    import torch
+    from oracle import hsc
+    prob, A, G, off, c, s = _cluster_and_plain(lib, monkeypatch, ne, M, p)
+    widths = [off[l + 1] - off[l] for l in range(p + 1)]
+    assert all(c.inner_path(w) in (1, 3) for w in widths) and all(s.inner_path(w) == 0 for w in widths)
+    lv = gmg.hierarchy(A[0], ne)
+    R = S.random_block(prob.n, c.P, seed=42)
+    o = lib.prec_opts(precision=lib.SG_F32, inner_fixed_iters=4)
+    Z, Z0 = (lib.hsc_precond_apply(h, torch.tensor(R, device="cuda"), o).cpu().numpy() for h in (c, s))
+
+    def dsolve(l, X):
+        return krylov.pcg_columns(lambda v: A[0] @ v, X, lambda r: gmg.vcycle(lv, r), tol=0.0, maxit=4,
+                                  fixed_iters=4)[0]
+    ref = hsc.hsc_apply(A, G, off, R, dsolve=dsolve)
+    tol = (1e-4 if ne == 64 else 2e-5) * np.abs(ref).max()
+    assert np.abs(Z - ref).max() <= tol and np.abs(Z - Z0).max() <= tol
+
+
+def test_solve_on_clusters(lib, monkeypatch):
+    """The mixed solve with its inner solves on the clusters reaches 1e-8 and
+    the oracle's direct solution."""
+    import torch
+    from oracle import sg_operator as so
+    prob, A, G, _, c, _ = _cluster_and_plain(lib, monkeypatch, 16, 3, 3)
+    F = S.make_rhs(prob, 3)
+    ref = so.direct_solve(A, G, F)
+    U, st = lib.sg_solve(c, torch.tensor(F, device="cuda"),
+                         lib.solve_opts(lib.prec_opts(precision=lib.SG_F32), precond=lib.SG_PREC_HSC, tol=1e-8))
+    assert st.true_rel_res <= 1e-8 * 1.01
+    assert np.abs(U.cpu().numpy() - ref).max() <= 1e-6 * np.abs(ref).max()
 
 
 @pytest.mark.parametrize("nu,omega", [(2, 0.8), (1, 0.8), (3, 0.7)])
