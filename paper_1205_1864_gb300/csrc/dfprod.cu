@@ -347,7 +347,7 @@ static int launch_df(sg_problem* h, const EdgeList& E, const TX* X, int ldx, int
   const size_t smem = df_smem(E, h->nterm, wx, DIAG);
   OuterArgs a = oa ? *oa : OuterArgs{};
   auto go = [&](auto kern) -> int {
-    SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(allow_smem(h, kern));
     int per_sm = 0;
     SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     int grid = std::min(h->n, h->num_sms * std::max(per_sm, 1));

@@ -1779,7 +1779,7 @@ static int launch_resid_restrict(sg_problem* h, const GridLevel& G, const GridLe
   const int bdim = std::min(1024, (items + 31) / 32 * 32);
   const size_t smem = (size_t)items * 16;
   auto tiles = [&](int t) { return ceil_div(C.nx, t) * ceil_div(C.ny, t); };
-  SG_TRY_CUDA(cudaFuncSetAttribute(k_resid_restrict_t<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SG_TRY(allow_smem(h, k_resid_restrict_t<T>));
   int per_sm = 0;
   SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_resid_restrict_t<T>, bdim, smem));
   const int grid = std::max(1, std::min(tiles(tc), h->num_sms * std::max(per_sm, 1)));

@@ -1168,17 +1168,6 @@ struct ClusterSolver {
   float4* wvecs = nullptr;    // k_inner_cluster_wide: r, p, x, A p
 };
 
-// Raise kern's dynamic shared-memory limit to at least `bytes`. The limit
-// belongs to the function, not to a problem: it is never lowered, so the plan
-// of one problem does not invalidate the launches of another.
-template <typename K>
-static bool allow_smem(K kern, unsigned bytes) {
-  cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return false;
-  if (fa.maxDynamicSharedSizeBytes >= (int)bytes) return true;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
-}
-
 // Clusters of `cln` CTAs of kernel kern resident at once with `bytes` of
 // dynamic shared memory (0 if it cannot run). Clusters of more than 8 CTAs
 // are a non-portable size the kernel has to opt in to.
@@ -1187,7 +1176,11 @@ static int max_clusters(K kern, unsigned bytes, int optin, int cln) {
   cudaFuncAttributes fa{};
   if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return 0;
   if ((long long)bytes + (long long)fa.sharedSizeBytes > optin) return 0;
-  if (!allow_smem(kern, bytes)) return 0;
+  // as allow_smem: the most a block may have, whatever this plan takes
+  const int most = optin - (int)fa.sharedSizeBytes;
+  if (fa.maxDynamicSharedSizeBytes < most &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
+    return 0;
   if (cln > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return 0;
   cudaLaunchConfig_t cfg = {};

@@ -399,7 +399,7 @@ static int launch_t(sg_problem* h, const TIn* X, int ldx, int wx, const EdgeList
     return SG_ERR_UNSUPPORTED;
   }
   auto go = [&](auto kern) -> int {
-    SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(allow_smem(h, kern));
     int per_sm = 0;
     SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     const int grid = std::min(h->n, h->num_sms * std::max(per_sm, 1));
@@ -490,7 +490,7 @@ static int launch_outer_t(sg_problem* h, const OuterArgs& a, cudaStream_t s) {
   const TAcc* vals = DF ? (const TAcc*)h->vals_df : (const TAcc*)h->vals64;
   const TAcc* ec = DF ? (const TAcc*)h->all.cdf : (const TAcc*)h->all.c64;
   auto go = [&](auto kern) -> int {
-    SG_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(allow_smem(h, kern));
     int per_sm = 0;
     SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     const int grid = std::min(std::min(h->n, h->num_sms * std::max(per_sm, 1)), h->opart_blocks);

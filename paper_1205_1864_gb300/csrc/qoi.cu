@@ -221,7 +221,7 @@ int sg_qoi_grad(sg_problem* h, const double* U, const double* Lam, int nparam, c
     return SG_ERR_UNSUPPORTED;
   }
   const size_t smem = (size_t)chunk * per_nz;
-  SG_TRY_CUDA(cudaFuncSetAttribute(k_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  SG_TRY(allow_smem(h, k_grad));
   int per_sm = 1;
   SG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_grad, 256, smem));
   const int grid = std::min(h->n, h->num_sms * std::max(per_sm, 1));
