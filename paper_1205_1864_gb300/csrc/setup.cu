@@ -74,7 +74,7 @@ __global__ void k_pack_stencil(int nx, int ny, const float* __restrict__ st, con
   }
 }
 
-int pack_stencils(GridLevel& g) {
+static int pack_stencils(GridLevel& g) {
   { k_pack_stencil<<<std::min((g.n * 12 + 255) / 256, 4096), 256>>>(g.nx, g.ny, g.st32, g.dinv32, g.st12, g.planes); ::sghsc::note_launch(); }
   SG_CHECK_LAUNCH();
   return SG_OK;
@@ -698,28 +698,36 @@ __global__ void k_scale_vals(long long count, int M1, const double* __restrict__
   }
 }
 
-// the V-cycle matrix of s * A_0: that of A_0 divided by s
-__global__ void k_scale_cmat(int n, const double* __restrict__ base, double s, double* __restrict__ m64,
-                             float* __restrict__ m32) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double v = base[i] / s;
-    m64[i] = v;
-    m32[i] = (float)v;
-  }
-}
-
-// multigrid stencils of s * A_0: st = s * base, dinv = 1 / (s * base_centre)
-__global__ void k_scale_grid(int n, const double* __restrict__ base, double s, double* __restrict__ st64,
-                             float* __restrict__ st32, double* __restrict__ dinv64, float* __restrict__ dinv32) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * 9; i += gridDim.x * blockDim.x) {
-    const double v = s * base[i];
-    st64[i] = v;
-    st32[i] = (float)v;
-    if (i % 9 == 4) {
-      dinv64[i / 9] = 1.0 / v;
-      dinv32[i / 9] = (float)(1.0 / v);
+// multigrid stencils of s * A_0: st = s * base, dinv = 1 / (s * base_centre),
+// and their FP32 copies (GridLevel::st12, planes; the padding stays as packed at
+// set-up). On the 7 x 7 grid also the V-cycle matrix, that of A_0 divided by s
+// (cbase: null elsewhere). One launch a grid: with the copies and the matrix in
+// launches of their own sg_set_scales took 52, 69 and 80 us on 15, 63 and 127
+// nodes a side, so 34, 42 and 50 (32, 40 and 48 without either).
+__global__ void k_scale_grid(GridLevel g, double s, const double* __restrict__ cbase, double* __restrict__ c64,
+                             float* __restrict__ c32) {
+  const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (int i = first; i < g.n * 9; i += step) {
+    const int node = i / 9, e = i - node * 9, x = node % g.nx, y = node / g.nx;
+    const double v = s * g.st_base[i];
+    g.st64[i] = v;
+    g.st32[i] = (float)v;
+    g.st12[node * 12 + e / 3 * 4 + e % 3] = (float)v;
+    if (g.planes) g.planes[(e * g.ny + y) * (g.nx + 1) + x] = (float)v;
+    if (e == 4) {
+      const double d = 1.0 / v;
+      g.dinv64[node] = d;
+      g.dinv32[node] = (float)d;
+      g.st12[node * 12 + 11] = (float)d;
+      if (g.planes) g.planes[(9 * g.ny + y) * (g.nx + 1) + x] = (float)d;
     }
   }
+  if (cbase)
+    for (int i = first; i < 49 * 49; i += step) {
+      const double v = cbase[i] / s;
+      c64[i] = v;
+      c32[i] = (float)v;
+    }
 }
 
 }  // namespace sghsc
@@ -748,11 +756,10 @@ int sg_set_scales(sg_problem* h, const double* scale) {
   SG_TRY_CUDA(cudaMemcpy(h->scales_dev, scale, h->nterm * sizeof(double), cudaMemcpyHostToDevice));
   const long long count = (long long)h->nnz * h->nterm;
   { k_scale_vals<<<(int)std::min<long long>((count + 255) / 256, 4096), 256>>>(count, h->nterm, h->vals_base, h->scales_dev, h->vals64, h->vals32, (df64*)h->vals_df); ::sghsc::note_launch(); }
-  for (auto& g : h->grids)
-    { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g.n, g.st_base, scale[0], g.st64, g.st32, g.dinv64, g.dinv32); ::sghsc::note_launch(); }
-  for (auto& g : h->grids) SG_TRY(pack_stencils(g));
-  if (h->cmat_base)
-    { k_scale_cmat<<<10, 256>>>(49 * 49, h->cmat_base, scale[0], h->cmat64, h->cmat32); ::sghsc::note_launch(); }
+  for (auto& g : h->grids) {
+    const double* cbase = h->cmat_base && &g == &h->grids[h->grids.size() - 3] ? h->cmat_base : nullptr;
+    { k_scale_grid<<<std::min((g.n * 9 + 255) / 256, 4096), 256>>>(g, scale[0], cbase, h->cmat64, h->cmat32); ::sghsc::note_launch(); }
+  }
   SG_TRY_CUDA(cudaGetLastError());
   SG_TRY_CUDA(cudaDeviceSynchronize());
   return SG_OK;

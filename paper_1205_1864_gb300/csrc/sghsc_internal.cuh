@@ -315,9 +315,6 @@ inline int allow_smem(const sg_problem* h, K* kern) {
   return SG_OK;
 }
 
-// The FP32 stencil copies of a grid (st12, planes) from st32 and dinv32.
-int pack_stencils(GridLevel& g);
-
 // ---- inner solver (inner.cu) ----
 int ensure_inner_work(sg_problem* h, int dtype, int wcap);
 void free_inner_work(sg_problem* h);
