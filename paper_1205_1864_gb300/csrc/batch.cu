@@ -245,13 +245,16 @@ static int autotune_outer(sg_problem* h, cudaStream_t s, bool df) {
 }
 
 // Tuned shapes per problem class: problems with the same device, sizes, chaos
-// space and row lengths run the same launches, so a class is timed once per
-// process and later handles of that class take its shapes without timing.
+// space, row lengths and kernels to choose from run the same launches, so a
+// class is timed once per process and later handles of that class take its
+// shapes without timing. solvers: the switches of the handle's environment that
+// leave kernels out, and the cluster solvers that it holds (a pick of 0 is the
+// block solver, or the stand-alone kernels, row-pipelined or not).
 struct TuneKey {
-  int dev, n, nnz, M, p, family, max_row, q, staged;
+  int dev, n, nnz, M, p, family, max_row, q, staged, solvers;
   bool operator<(const TuneKey& o) const {
-    return std::tie(dev, n, nnz, M, p, family, max_row, q, staged) <
-           std::tie(o.dev, o.n, o.nnz, o.M, o.p, o.family, o.max_row, o.q, o.staged);
+    return std::tie(dev, n, nnz, M, p, family, max_row, q, staged, solvers) <
+           std::tie(o.dev, o.n, o.nnz, o.M, o.p, o.family, o.max_row, o.q, o.staged, o.solvers);
   }
 };
 struct TuneVal {
@@ -262,7 +265,9 @@ static std::mutex g_tune_mu;
 static std::map<TuneKey, TuneVal> g_tune_cache;
 
 static TuneKey tune_key(const sg_problem* h) {
-  return TuneKey{h->device, h->n, h->nnz, h->M, h->p, h->family, h->max_row_nnz, h->q, h->staged_pairs};
+  int solvers = (h->block_off ? 1 : 0) | (h->pipe_off ? 2 : 0);
+  for (int path : inner_path_candidates(h, 1)) solvers |= 4 << path;
+  return TuneKey{h->device, h->n, h->nnz, h->M, h->p, h->family, h->max_row_nnz, h->q, h->staged_pairs, solvers};
 }
 
 // A block size the product kernels are instantiated for: whole warps, 32 to
