@@ -235,7 +235,8 @@ int sg_apply(sg_problem* h, const void* U, void* Y, int dtype, void* stream);
  * w_d = number of chaos polynomials of degree d. dtype SG_F64 or SG_F32 for
  * all three blocks, or SG_F32_ACC64 / SG_F32_ACCDF64: X and Yout FP32, Yin
  * FP64 (required, not aliasing Yout), the sum accumulated in FP64 or in
- * double-float arithmetic. */
+ * double-float arithmetic. On a handle of sg_setup_gpc only levels 0 and 1
+ * (SG_ERR_UNSUPPORTED else: its level products reach all lower levels). */
 int sg_level_apply(sg_problem* h, int lvl_out, int lvl_in, const void* X, const void* Yin,
                    void* Yout, int dtype, void* stream);
 

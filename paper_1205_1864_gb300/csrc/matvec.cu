@@ -549,6 +549,10 @@ int sg_level_apply(sg_problem* h, int lvl_out, int lvl_in, const void* X, const 
   const EdgeList& E = lvl_in > lvl_out ? h->pre[lvl_in] : h->post[lvl_out];
   const int win = h->off[lvl_in + 1] - h->off[lvl_in];
   const int wout = h->off[lvl_out + 1] - h->off[lvl_out];
+  if (E.nin != win || E.nout != wout) {   // gPC: the list reaches every lower level, the blocks hold one
+    set_error("sg_level_apply: a gPC coefficient couples level %d to all lower levels", std::max(lvl_in, lvl_out));
+    return SG_ERR_UNSUPPORTED;
+  }
   if (mixed)   // the level-p products of the mixed preconditioner with an FP64-accurate top level
     return launch_block_matvec(h, SG_F32, dtype == SG_F32_ACC64 ? SG_F64 : ACC_DF64, SG_F64, SG_F32, X, win, win, E,
                                false, Yin, wout, -1.0, 1.0, Yout, wout, (cudaStream_t)stream);
