@@ -140,19 +140,15 @@ static Shape fit(const sg_problem* h, Shape s, K kern) {
   return s;
 }
 
-// Width of a batch of w columns in the workspace: whole 16-byte pieces, and
-// from 97 FP32 columns on whole 128-byte lines, so that a strip's part of a
-// node is one line and not parts of two (as long as n times the width stays
-// within 32 bits).
+// Width of a batch of w columns in the workspace: whole 16-byte pieces. (Whole
+// 128-byte lines from 97 columns on, a strip's part of a node one line and not
+// parts of two, were slower: six steps on 255 x 255 nodes, 97 columns, 1695
+// against 1609 us, 129 columns 1979 against 1863; 127 x 127, 161 columns, 971
+// against 917; equal from 481 columns on.)
 template <typename T>
-static int vector_width(int w) {
+static int padded_width(int w) {
   constexpr int N = 16 / (int)sizeof(T);
   return (w + N - 1) / N * N;
-}
-template <typename T>
-static int padded_width(int w, int n) {
-  const int lines = (w + 31) / 32 * 32;
-  return sizeof(T) == 4 && w > 96 && (long long)n * lines < (1LL << 31) ? lines : vector_width<T>(w);
 }
 
 enum { FIN_INIT = 0, FIN_RHO = 1, FIN_ALPHA = 2, FIN_CONV = 3 };
@@ -1664,7 +1660,7 @@ int ensure_inner_work(sg_problem* h, int dtype, int wcap) {
     return SG_ERR_UNSUPPORTED;
   }
   InnerWork& iw = dtype == SG_F64 ? h->iw64 : h->iw32;
-  wcap = std::max((wcap + 3) / 4 * 4, padded_width<float>(wcap, h->grids[0].n));   // room for either precision
+  wcap = (wcap + 3) / 4 * 4;   // room for the padded width of either precision
   if (iw.wcap >= wcap) return SG_OK;
   if (h->capturing) {
     set_error("inner solve: workspace must be allocated before graph capture");
@@ -1920,7 +1916,7 @@ static int inner_solve_t(sg_problem* h, const void* src, int ld_src, int src_t, 
   constexpr int N = VW<T>::N;
   InnerWork& iw = sizeof(T) == 8 ? h->iw64 : h->iw32;
   const GridLevel& G = h->grids[0];
-  const int wp = padded_width<T>(w, G.n), ng = wp / N;
+  const int wp = padded_width<T>(w), ng = wp / N;
   const Shape sh = make_shape(h, G.n, ng, 1);    // gather / matvec / update end in reductions
   T* x = (T*)iw.x;
   T* r = (T*)iw.r;
@@ -1988,10 +1984,11 @@ int inner_solve(sg_problem* h, int dtype, const void* src, int ld_src, int src_t
 // packed into the padded workspace, the cycle runs there, the result is
 // unpacked into X.
 template <typename T>
-static int vcycle_packed(sg_problem* h, InnerWork& iw, const T* B, T* bpad, T* X, int w, int wp,
-                         const sg_prec_opts& o, cudaStream_t s) {
+static int vcycle_packed(sg_problem* h, InnerWork& iw, const T* B, T* bpad, T* X, int w, const sg_prec_opts& o,
+                         cudaStream_t s) {
   constexpr int N = VW<T>::N;
   const GridLevel& G = h->grids[0];
+  const int wp = padded_width<T>(w);
   const Shape sh = make_shape(h, G.n, wp / N);
   { k_pack<T, T><<<sh.grid, sh.bdim, 0, s>>>(G.n, w, wp, sh.k, B, w, bpad); ::sghsc::note_launch(); }
   const T* res = nullptr;
@@ -2010,7 +2007,7 @@ static int m0_apply_t(sg_problem* h, const T* src, int lds, T* dst, int ldd, int
   constexpr int N = VW<T>::N;
   InnerWork& iw = sizeof(T) == 8 ? h->iw64 : h->iw32;
   const GridLevel& G = h->grids[0];
-  const int wp = padded_width<T>(w, G.n);
+  const int wp = padded_width<T>(w);
   const Shape sh = make_shape(h, G.n, wp / N);
   { k_clear_done<<<1, 1024, 0, s>>>(iw.wcap, iw.done); ::sghsc::note_launch(); }
   { k_pack<T, T><<<sh.grid, sh.bdim, 0, s>>>(G.n, w, wp, sh.k, src, lds, (T*)iw.r); ::sghsc::note_launch(); }
@@ -2038,11 +2035,8 @@ int inner_vcycle(sg_problem* h, int dtype, const void* B, void* X, int w, const 
   SG_TRY(ensure_inner_work(h, dtype, std::max(w, h->wmax)));
   InnerWork& iw = dtype == SG_F64 ? h->iw64 : h->iw32;
   { k_clear_done<<<1, 1024, 0, s>>>(iw.wcap, iw.done); ::sghsc::note_launch(); }
-  const int n = h->grids[0].n;
-  if (dtype == SG_F64)
-    return vcycle_packed<double>(h, iw, (const double*)B, (double*)iw.r, (double*)X, w, padded_width<double>(w, n), o,
-                                 s);
-  return vcycle_packed<float>(h, iw, (const float*)B, (float*)iw.r, (float*)X, w, padded_width<float>(w, n), o, s);
+  if (dtype == SG_F64) return vcycle_packed<double>(h, iw, (const double*)B, (double*)iw.r, (double*)X, w, o, s);
+  return vcycle_packed<float>(h, iw, (const float*)B, (float*)iw.r, (float*)X, w, o, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -2111,7 +2105,7 @@ int vcycle_static(sg_problem* h, int dtype, const void* B, void* X, int w, const
     return SG_ERR_UNSUPPORTED;
   }
   const size_t es = dtype == SG_F64 ? 8 : 4;
-  const int wp = dtype == SG_F64 ? vector_width<double>(w) : vector_width<float>(w);
+  const int wp = dtype == SG_F64 ? padded_width<double>(w) : padded_width<float>(w);
   const size_t need = static_vcycle_bytes(h, wp, es);
   if (need > STATIC_SCRATCH_BYTES) {
     set_error("sg_vcycle_apply_static: %d columns of %d nodes need %zu bytes of scratch, above the fixed %zu",
@@ -2147,8 +2141,8 @@ int vcycle_static(sg_problem* h, int dtype, const void* B, void* X, int w, const
   }
   // the kernels skip columns whose done flag is set: start from all zero
   SG_TRY_CUDA(cudaMemsetAsync(sw.done, 0, (size_t)wp * sizeof(int), s));
-  if (dtype == SG_F64) return vcycle_packed<double>(h, sw, (const double*)B, (double*)sw.r, (double*)X, w, wp, o, s);
-  return vcycle_packed<float>(h, sw, (const float*)B, (float*)sw.r, (float*)X, w, wp, o, s);
+  if (dtype == SG_F64) return vcycle_packed<double>(h, sw, (const double*)B, (double*)sw.r, (double*)X, w, o, s);
+  return vcycle_packed<float>(h, sw, (const float*)B, (float*)sw.r, (float*)X, w, o, s);
 }
 
 }  // namespace sghsc
