@@ -131,9 +131,10 @@ static int batch_solve(sg_batch* b, const double* const* F, double* const* U, co
 
 // Candidate block sizes of the full product: powers of two from 64 to 1024 and
 // the whole-warp sizes that give every thread 1, 2 or 4 outputs with at most
-// 31 idle lanes (224 for P = 210).
-static std::vector<int> block_candidates(int P) {
+// 31 idle lanes (224 for P = 210; not with powers_only).
+static std::vector<int> block_candidates(int P, bool powers_only = false) {
   std::vector<int> c = {64, 128, 256, 512, 1024};
+  if (powers_only) return c;
   for (int m : {1, 2, 4}) {
     const int t = 32 * ceil_div(P, 32 * m);
     if (t >= 64 && t <= 1024 && std::find(c.begin(), c.end(), t) == c.end()) c.push_back(t);
@@ -143,8 +144,7 @@ static std::vector<int> block_candidates(int P) {
 
 // Time the full SG product with each candidate block size, in pair and in
 // gather form, and keep the fastest.
-// whole_warps: the sizes beside the powers of two too.
-static int autotune_k1(sg_problem* h, int dtype, bool whole_warps, cudaStream_t s) {
+static int autotune_k1(sg_problem* h, int dtype, bool powers_only, cudaStream_t s) {
   const size_t es = dtype == SG_F64 ? 8 : 4;
   const size_t bytes = (size_t)h->n * h->P * es;
   void *X = nullptr, *Y = nullptr;
@@ -158,8 +158,7 @@ static int autotune_k1(sg_problem* h, int dtype, bool whole_warps, cudaStream_t 
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  std::vector<int> cands = block_candidates(h->P);
-  if (!whole_warps) cands.resize(5);
+  const std::vector<int> cands = block_candidates(h->P, powers_only);
   const int nc = (int)cands.size();
   int best = 0, best_pairs = 1;
   float best_ms = 1e30f;
@@ -377,16 +376,17 @@ int sg_autotune(sg_problem* h, void* stream) {
       return SG_OK;
     }
   }
-  SG_TRY(autotune_k1(h, SG_F64, true, (cudaStream_t)stream));
-  // the FP32 full product takes the row kernel (fixed shape) where it applies; up
-  // to 511 columns the general kernel's shape is still tuned and reported, for
-  // the forms that the row kernel does not take: it is the general kernel that
-  // is timed, over the powers of two
+  SG_TRY(autotune_k1(h, SG_F64, false, (cudaStream_t)stream));
+  // where the row kernel (fixed shape) takes the FP32 full product it is not
+  // timed. Up to 511 columns sg_autotune_result reports the general kernel's
+  // shape all the same, as it always has; only the general double-float product,
+  // should it stand in, launches with it. Powers of two only: for P = 84 the 96
+  // threads between two of them were within the noise of 64 and 128
   const bool row_kernel = rows32_usable(h, h->all, h->P, true);
   if (h->P < 512 || !row_kernel) {
     const int staged = h->staged_pairs;
     h->staged_pairs = 0;
-    const int r = autotune_k1(h, SG_F32, !row_kernel, (cudaStream_t)stream);
+    const int r = autotune_k1(h, SG_F32, row_kernel, (cudaStream_t)stream);
     h->staged_pairs = staged;
     SG_TRY(r);
   }
