@@ -253,8 +253,7 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
       df64 acc(0.f, 0.f);
       if (re > rb) {
         if (DIAG) acc = df64(Dh[l], Dl[l]);
-        // two couplings at a time, side by side in packed sums; past the last
-        // one the zero coefficient class (word 0)
+        // two couplings at a time, side by side in packed sums (the counts are even)
         auto at = [](const float* p, unsigned byte) {
           return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(p) + byte);
         };
@@ -276,7 +275,7 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
           couple(w0, w1, s);
           couple(w2, w3, s);
         }
-        for (; c < ncl; c += 2, cw += 64) couple(__ldg(cw), c + 1 < ncl ? __ldg(cw + 32) : 0u, s);
+        for (; c < ncl; c += 2, cw += 64) couple(__ldg(cw), __ldg(cw + 32), s);
         acc += df64(s.hi.x, s.lo.x);
         acc += df64(s.hi.y, s.lo.y);
       }
@@ -317,8 +316,8 @@ __global__ void __launch_bounds__(LB, LB <= 256 ? 4 : 2) k_df_pairs(
   }
 }
 
-// Block size: 256 threads when every thread's pairs fit its registers, else
-// 512 (more, smaller blocks hide the row barriers better).
+// Block size: 256 threads up to DF_MAXQ pairs a thread, else 512 (more, smaller
+// blocks hide the row barriers better).
 static int df_threads(const EdgeList& E) { return E.npair <= DF_MAXQ * 256 ? 256 : 512; }
 
 // (at least the outer step's final sums of two doubles per thread)

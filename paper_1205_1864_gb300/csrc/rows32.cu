@@ -78,11 +78,12 @@ __global__ void __launch_bounds__(rows32::NT, 4) k_rows32(
   const int wts = (wx + PASS - 1) / PASS * PASS;   // rows32_stride
   float* Ctab = reinterpret_cast<float*>(sm4);                        // [ncls]
   float4* Vall = sm4 + (ncls + 3) / 4;                                 // [ROWS][M1][VS4]
-  float* Tall = reinterpret_cast<float*>(Vall + (size_t)ROWS * M1 * VS4);   // [ROWS][M1][wts]
+  float* Tall = reinterpret_cast<float*>(Vall + (size_t)ROWS * M1 * VS4);   // [ROWS]: [M1][wts], zero (padding couplings)
   const int tid = threadIdx.x, g = tid / RG, lt = tid - g * RG;
   float4* Vt = Vall + (size_t)g * M1 * VS4;
   float* Vf = reinterpret_cast<float*>(Vt);
-  float* Ts = Tall + (size_t)g * M1 * wts;
+  float* Ts = Tall + (size_t)g * (M1 * wts + 4);
+  if (lt == 0) Ts[M1 * wts] = 0.f;
   for (int t = tid; t < ncls; t += NT) Ctab[t] = ctab[t];
   for (long long rbase = (long long)blockIdx.x * ROWS; rbase < n; rbase += (long long)gridDim.x * ROWS) {
     const int r = (int)rbase + g;

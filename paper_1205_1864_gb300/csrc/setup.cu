@@ -187,8 +187,8 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0, int in0, int
     if (fits && pk.size() < (1u << 20)) SG_TRY(upload(&E.pkj, w.data(), w.size()));
   }
   {
-    // coefficient classes; class 0 is the coefficient 0, which pads the
-    // shorter slots of a warp to the warp's longest (a zero word adds 0)
+    // coefficient classes; class 0 is the coefficient 0, which pads the shorter
+    // slots of a warp to the warp's longest
     std::map<double, int> cls;
     for (double c : he.c) cls.emplace(c, 0);
     if (cls.size() + (cls.count(0.0) ? 0 : 1) <= 256 && E.npair < (1 << 24)) {
@@ -202,21 +202,22 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0, int in0, int
       }
       SG_TRY(upload(&E.ctab32, tab32.data(), tab32.size()));
       // slot-transposed packing: warp w (slots 32w .. 32w+31, counts sorted
-      // descending) takes 32 words per coupling of its first slot
+      // descending) takes 32 words per coupling of its first slot, and 32 more
+      // for an even number
+      auto steps = [&](int sl) { return (he.ptr[perm[sl & ~31] + 1] - he.ptr[perm[sl & ~31]] + 1) & ~1; };
       std::vector<int> tb(E.nout);
       size_t total = 0;
       for (int w0 = 0; w0 < E.nout; w0 += 32) {
-        const int cmax = he.ptr[perm[w0] + 1] - he.ptr[perm[w0]];
+        const int cmax = steps(w0);
         for (int sl = w0; sl < std::min(w0 + 32, E.nout); ++sl) tb[sl] = (int)total + (sl - w0);
         total += (size_t)32 * cmax;
       }
       if (total >= (size_t)1 << 31) return SG_ERR_UNSUPPORTED;
       std::vector<unsigned> packed(std::max<size_t>(total, 1), 0u), pkj;
-      bool kj_ok = true;
       E.rows32 = rows32_rows(nin, E.nout, nin == E.nout && in0 == out0, terms);
       const int wts = rows32_stride(nin, E.rows32);   // the row stride of the FP32 row kernel's term sums
-      for (int t = 0; t < E.nedges; ++t) kj_ok = kj_ok && (long long)he.k[t] * wts + he.j[t] < (1 << 24);
-      if (kj_ok) pkj.assign(packed.size(), 0u);
+      const bool kj_ok = (long long)terms * wts < (1 << 24);
+      if (kj_ok) pkj.assign(packed.size(), (unsigned)(terms * wts));
       std::vector<unsigned> cof(E.nedges);
       for (int t = 0; t < E.nedges; ++t) cof[t] = (unsigned)cls.at(he.c[t]);
       for (int w0 = 0; w0 < E.nout; w0 += 32) {
@@ -232,21 +233,20 @@ static int upload_edges(const HostEdges& he, EdgeList& E, int out0, int in0, int
           }
         }
         const std::vector<int> ss = schedule_warp(as, ws);
-        for (size_t c = 0; c < ss.size() / 32; ++c)
-          for (int i = 0; i < ws; ++i) {   // padding stays the zero word
-            const int qs = ss[c * 32 + i];
-            if (qs >= 0) packed[(size_t)tb[w0 + i] + 32 * c] = ((unsigned)as[i][qs] << 12) | cof[he.ptr[perm[w0 + i]] + qs] << 2;
+        for (int c = 0; c < steps(w0); ++c)
+          for (int i = 0; i < ws; ++i) {
+            const int qs = (size_t)c * 32 < ss.size() ? ss[c * 32 + i] : -1, own = as[i].empty() ? 0 : as[i][0];
+            packed[(size_t)tb[w0 + i] + 32 * c] =
+                qs < 0 ? (unsigned)own << 12 : (unsigned)as[i][qs] << 12 | cof[he.ptr[perm[w0 + i]] + qs] << 2;
           }
       }
       if (E.nout < 65536) {
-        // per slot: its first word and (output << 16 | couplings of the
-        // warp's longest slot, the others padded with zero words), so the
+        // per slot: its first word and (output << 16 | steps of its warp), so the
         // lanes of a warp run the same coupling loop
         std::vector<int2> sd(E.nout);
         bool ok = true;
         for (int sl = 0; sl < E.nout; ++sl) {
-          const int l = perm[sl], l0 = perm[sl & ~31];
-          const int cnt = he.ptr[l0 + 1] - he.ptr[l0];
+          const int l = perm[sl], cnt = steps(sl);
           ok = ok && cnt < 65536;
           sd[sl] = make_int2(tb[sl], (int)(((unsigned)l << 16) | (unsigned)cnt));
         }

@@ -80,13 +80,14 @@ struct EdgeList {
   // lanes of a warp (32 consecutive slots) read consecutive words; tb(s) is in
   // the slot's descriptor (sdesc). The order of an output's couplings over the
   // steps is chosen per warp so that their sums lie in different shared-memory
-  // banks.
+  // banks. The shorter slots of a warp are padded with the coefficient 0 times a
+  // sum of their own (another's could be infinite), to an even number of steps.
   unsigned* ctr = nullptr;
   // the pairs as staged offsets of the double-float products, k DF_VS << 16 | j DF_XS
   // (null when one does not fit 16 bits)
   unsigned* pkj = nullptr;
   // the same for the FP32 row kernel, in list order: class << 24 | (k
-  // rows32_stride(nin, rows32) + j) (below 2^24)
+  // rows32_stride(nin, rows32) + j) (below 2^24), padding at the zero behind the sums
   unsigned* ckj = nullptr;
   int rows32 = 0;            // rows per block of that kernel (0: not taken)
   int2* sdesc = nullptr;     // per slot: tb(s), output << 16 | steps of its warp
@@ -295,7 +296,7 @@ __host__ __device__ constexpr int rows32_stride(int wx, int rows) {
   return (wx + pass - 1) / pass * pass;
 }
 constexpr size_t rows32_smem(int ncls, int terms, int wx, int rows) {
-  return (size_t)((ncls + 3) & ~3) * 4 + (size_t)rows * terms * (48 + (size_t)rows32_stride(wx, rows) * 4);
+  return (size_t)((ncls + 3) & ~3) * 4 + (size_t)rows * (terms * (48 + (size_t)rows32_stride(wx, rows) * 4) + 16);
 }
 // FP32 products with the input columns in registers (rows32.cu): usable and
 // preferred for E (compact table, sizes).
