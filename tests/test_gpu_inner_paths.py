@@ -122,3 +122,26 @@ def test_coarse_matrix_in_the_fp32_block_solver(lib, monkeypatch, ne):
     X = [lib.sg_inner_solve(h, B, lib.prec_opts(precision=lib.SG_F32, inner_fixed_iters=1, omega=om))[0]
          for om in (0.8, float(np.nextafter(0.8, 1)))]
     assert float((X[0] - X[1]).abs().max()) <= 1e-5 * float(X[1].abs().max())
+
+
+@pytest.mark.parametrize("ne,w,prec", [(16, 6, "fp64"), (32, 5, "fp64"), (16, 6, "fp32"), (32, 5, "fp32"), (64, 7, "fp32")])
+@pytest.mark.parametrize("nu,omega", [(1, 0.8), (3, 0.7), (2, 0.6)])
+def test_block_solver_with_other_smoothing(lib, monkeypatch, ne, w, prec, nu, omega):
+    """The block solver alone, grid by grid (no coarse matrix), odd and even
+    numbers of sweeps: three steps against the oracle, 1e-11 of the largest entry
+    in FP64, 1e-4 in FP32."""
+    import torch
+    prob, A, _, _ = problem(ne, 1, 1)
+    monkeypatch.setenv("SGHSC_NO_CLUSTER", "1")
+    h = lib.SGProblem.from_inputs(prob, 1)
+    code, dt, tol = (lib.SG_F64, np.float64, 1e-11) if prec == "fp64" else (lib.SG_F32, np.float32, 1e-4)
+    lv = gmg.hierarchy(A[0], ne)
+    B = S.random_block(prob.n, w, seed=ne + nu).astype(dt)
+    n0 = lib._lib.LIB.sg_kernel_launches()
+    X, it = lib.sg_inner_solve(h, torch.tensor(B, device="cuda"),
+                               lib.prec_opts(precision=code, inner_fixed_iters=3, nu=nu, omega=omega))
+    assert lib._lib.LIB.sg_kernel_launches() - n0 == 1
+    ref = krylov.pcg_columns(lambda v: A[0] @ v, B.astype(np.float64), lambda r: gmg.vcycle(lv, r, nu=nu, omega=omega),
+                             tol=0.0, maxit=3, fixed_iters=3)[0]
+    assert list(it) == [3] * w
+    assert np.abs(X.double().cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
