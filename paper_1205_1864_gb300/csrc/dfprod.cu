@@ -11,8 +11,8 @@
 //           lanes of a warp (consecutive pairs: the same k, consecutive j)
 //           read one broadcast value and 32 distinct banks (stride 9 words);
 //   pairs   every distinct (k, j) of the couplings: S_q = sum_e a_k(e) X(e, j)
-//           into shared memory, each thread keeping its pairs in registers;
-//           with DIAG also the k = 0 term of its own outputs;
+//           into shared memory, a thread reading its pairs' offsets one turn
+//           ahead; with DIAG also the k = 0 term of its own outputs;
 //   couple  Y(r, l) = diag + sum_t c_t S_pair(t) over the couplings of l.
 // Rows longer than CH are done in chunks of CH (the first chunk stores, later
 // ones add).
@@ -26,7 +26,7 @@
 namespace sghsc {
 
 constexpr int DF_CH = 9;       // nonzeros per staged chunk (the Q1 stencil row)
-constexpr int DF_MAXQ = 12;    // pairs per thread and row at most
+constexpr int DF_MAXQ = 12;    // pairs per thread and row at most (what was measured: the sums are in shared memory)
 
 // FP32 value of an input element that is FP32-exact: a float as it is, a
 // double (the FP64 widening of an FP32 number) re-packed with integer
@@ -329,9 +329,9 @@ static size_t df_smem(const EdgeList& E, int M1, int wx, bool diag) {
                   t * 2 * sizeof(double));
 }
 
-// Usable when every thread's pairs fit its registers, the couplings have a
-// compact table with slot descriptors and the staging fits a block's shared
-// memory.
+// Usable up to DF_MAXQ pairs for each of 512 threads (beyond, the general
+// kernel), when the couplings have a compact table with slot descriptors, the
+// pairs' offsets fit 16 bits and sums and staging fit a block's shared memory.
 bool df_pairs_usable(const sg_problem* h, const EdgeList& E, int wx) {
   return h->staged_pairs && E.npair <= DF_MAXQ * 512 && (E.pkj || E.npair == 0) && E.ncls > 0 && E.sdesc && h->nterm * DF_VS < 65536 &&
          wx * DF_XS < 65536 && df_smem(E, h->nterm, wx, true) + 4 * 1024 <= (size_t)std::max(h->smem_optin, 48 * 1024);

@@ -1560,7 +1560,9 @@ __global__ void __launch_bounds__(pipe::NT, 1)
 // kernel-per-sweep: 127 x 127 x 4 columns 97 against 189 us, x 330 222
 // against 251, x 126 (not taken) 159 against 135; 255 x 255 x 20 154 against
 // 175, x 330 478 against 679; 511 x 511 x 36 323 against 377, x 715 2761
-// against 4433 us.
+// against 4433 us. From 200,000 nodes every width is taken; 40 columns is where
+// the narrow strips give way: 511 x 511 x 40 333 against 394, x 44 (wide) 373
+// against 406; 1023 x 1023 x 40 854 against 1186, x 44 990 against 1183.
 static bool fused_narrow(const GridLevel& G, int wp) { return wp <= (G.n >= 200000 ? 40 : 24); }
 template <typename T>
 static bool use_fused(const sg_problem* h, const GridLevel& G, const GridLevel& C, int wp, const sg_prec_opts& o) {

@@ -34,11 +34,12 @@
 //
 // Measured against the stand-alone kernels, sg_inner_solve with its copies
 // and synchronisation, 20 steps of the diagonal M_0 or 2 of the V-cycle:
-// 29 x 29 nodes, FP64, 20 columns 1412 -> 159 us, 1000 columns 4584 -> 1029;
-// 63 x 63, FP64, 300 columns 2833 -> 1503; 9 x 9, 20 columns 1487 -> 143;
-// V-cycle 15 x 15, FP64, 20 columns 251 -> 104 (since then the matrix and the
-// staging below), 31 x 31, FP32, 300 columns 229 -> 120. No size it can hold was slower (1 to 1000 columns, both
-// types), so every batch that fits takes it. Whole FP64 solves: 16 x 16
+// 29 x 29 nodes, FP64, 20 columns 1284 -> 154 us, 1000 columns 4724 -> 1021;
+// 63 x 63, FP64, 300 columns 2824 -> 1502; 9 x 9, 20 columns 1288 -> 127;
+// V-cycle 15 x 15, FP64, 20 columns 218 -> 91, 31 x 31, FP64, 20 columns 256 ->
+// 128, FP32, 300 columns 199 -> 105, 63 x 63, FP32, 300 columns 286 -> 146. No
+// size it can hold was slower (1 to 1000 columns, both types), so every batch
+// that fits takes it before the stand-alone kernels. Whole FP64 solves: 16 x 16
 // elements, M = 3, p = 3, 6.64 -> 1.30 ms; 30 x 30, diagonal M_0, M = 4, p = 4,
 // 274 -> 15.4 ms; lognormal 10 x 10, M = 3, p = 3, 1034 -> 77.6 ms.
 #include <cooperative_groups.h>
@@ -702,8 +703,11 @@ __global__ void __launch_bounds__(blk::CNT) k_vcycle_coarse(BlockGrids L, int g0
 // and 32 + 4 s .. of row y: a row is read as two 16-byte pieces per thread, the
 // neighbours beside them come from the lanes beside it. The coarse grids run
 // in shared memory through block_vcycle. What bounds it: the barriers and the
-// chains between them (a step is 12.5 us, half of it on the coarse grids). Read node by node, the stencils took 4 us of a solve of two steps;
-// from planes with rows of 64 they are whole lines.
+// chains between them (a step is 12.5 us, half of it on the coarse grids; 35% of
+// the issue slots used, a warp waiting 2.6 clocks for shared memory and 2.0 at
+// barriers of 11.2 between two instructions). Read node by node, the stencils
+// took 4 us of a solve of two steps; from planes with rows of 64 they are whole
+// lines.
 namespace blk63 {
 constexpr int NT = 512, NX = 63;
 constexpr int W = 72;                 // row stride: node x at 4 + x, zeros around

@@ -23,13 +23,17 @@
 // zero-filled, the diagonal included, so no value needs a test: outside nodes
 // stay zero.
 //
-// What bounds it: instruction issue and the block's barrier per row (17 warps on
-// an SM: the rings take its shared memory); DRAM moves a quarter of its rate. At
-// 255 x 255 x 716 columns the four kernels this replaces took 135 + 180 + 234 +
-// 163 us, these two 150 + 253; a V-cycle 1245 -> 830 us, at 511 x 511
-// 4433 -> 2761 us. Tried: b's own values of five rows in registers (spills at
-// 96 registers a thread doubled the time of the way up), rows of b on 64-byte
-// instead of 128-byte boundaries (a third more DRAM reads).
+// What bounds it: instruction issue. At 255 x 255 x 716 columns 62% of the issue
+// slots are used by the 17 warps that an SM holds (the rings take its shared
+// memory); a warp's wait between two instructions, 6.8 clocks, is shared-memory
+// latency (1.8), another warp chosen (1.2) and the block's barrier per row
+// (1.0). 290 and 440 instructions a thread and row on the way down and up, a
+// quarter of them the stencils' multiply-adds; DRAM moves 35% of its rate. The
+// four kernels this replaces took 135 + 180 + 234 + 163 us, these two 157 + 256;
+// a V-cycle 1245 -> 830 us, at 511 x 511 4433 -> 2761 us. Tried: b's own values
+// of five rows in registers (spills at 96 registers a thread doubled the time of
+// the way up), rows of b on whole 128-byte lines (46% and 31% fewer bytes from
+// DRAM, the same time, and the padding cost every other kernel: inner.cu).
 //
 // Nodes x0 - 2 .. x0 + 65 (68 lanes) carry the two nodes a side that the last
 // sweep's neighbours need. A run of rows starts three rows early and ends five
@@ -387,8 +391,10 @@ __global__ void __launch_bounds__(mg::LX * PG, 1)
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();   // the rings are free
     if (DOT) {
-      // the strip's sums per column, nodes in order (the rows' buffers hold
-      // nothing needed any more; zero again for the next strip's first steps)
+      // the strip's sums per column, nodes in order. They overwrite rows of b:
+      // the next strip's copies fill every row that it reads of those. (What the
+      // buffers of x and y still hold goes only into the rows formed before the
+      // run's own, which nothing reads.)
       float* red = reinterpret_cast<float*>(R.br);   // [LX][4 PG]
       reinterpret_cast<float4*>(red)[lx * PG + grp] = acc;
       __syncthreads();
